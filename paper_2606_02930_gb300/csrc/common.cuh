@@ -50,6 +50,7 @@ struct GemmArgs {
   cplx* C; long long ldc, sCb;
   cplx alpha, beta;
   const cplx* Z; cplx gamma;   // optional: C = alpha*AB + beta*C + gamma*Z
+  const int* run_if = nullptr; // optional device word: nothing is computed when it is 0
 };
 cudaError_t zgemm(const GemmArgs& g, cudaStream_t st);
 
@@ -210,6 +211,39 @@ cudaError_t lq_formq(const cplx* W, const double* refl, int q, int k, cplx* Qh,
                      unsigned int* dev_state, cudaStream_t st);
 // R (k x p, k = min(p, q)) = L^H from the output of svd_lq
 cudaError_t svd_lq_r(const cplx* W, const cplx* beta, int p, int q, cplx* R, cudaStream_t st);
+// Preconditioner of the Jacobi (svd_pre.cu): its workspace for a k x p factor R
+// and the steps between the GEMMs, which the engine issues.  K[0..3] are k x k
+// matrices; ok, gate_n, gate, gate_w, gate_w2 are device words for GemmArgs::run_if
+// (V usable; a third Newton-Schulz step needed; a correction E to apply; its
+// square, its fourth power needed); err
+// is nonzero after a bounded wait ran out; act lists the rows left to the FP64
+// Jacobi (as jacobi_rows takes them).
+struct SvdPre {
+  void* rows32;
+  cplx* K[4];
+  int *act, *ok, *gate_n, *gate, *gate_w, *gate_w2, *err;
+  unsigned int* ctl;
+};
+size_t svd_pre_bytes(int k, int p);
+SvdPre svd_pre_carve(void* ws, int k, int p);
+// K[0] = V (k x k) from the fp32 block Jacobi on the rows of R; clears the
+// control words.  One cooperative launch of clusters.
+cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const double* anorm2,
+                           cudaStream_t st);
+// M = V V^H (k x k) becomes -(M - I) / 2; step 0 decides *ok, step 1 *gate_n
+cudaError_t svd_pre_orth(const SvdPre& s, cplx* M, int k, int step, cudaStream_t st);
+// E (k x k) from G = S S^H, and the gates
+cudaError_t svd_pre_corr(const SvdPre& s, const cplx* G, int k, double tol, const double* anorm2,
+                         double skip_rel, cplx* E, cudaStream_t st);
+// E += W / 2 - W2 / 8 as the gates say
+cudaError_t svd_pre_comb(const SvdPre& s, cplx* E, const cplx* W, const cplx* W2, int k,
+                         cudaStream_t st);
+// act from G = S S^H
+cudaError_t svd_pre_list(const SvdPre& s, const cplx* G, int k, double tol, const double* anorm2,
+                         double skip_rel, cudaStream_t st);
+// y = x if (*flag != 0) == want
+cudaError_t vec_copy_if(cplx* y, const cplx* x, long long n, const int* flag, bool want,
+                        cudaStream_t st);
 // One-sided Jacobi on the rows (length len) of A until they are mutually
 // orthogonal; no rotation is accumulated.  One cooperative launch;
 // dev_state (24 device words) returns the sweeps done in word 5, the pairs
@@ -219,11 +253,12 @@ cudaError_t svd_lq_r(const cplx* W, const cplx* beta, int p, int q, cplx* R, cud
 // rows whose squared norms are both <= skip_rel |A|_F^2 are left as they are.
 // keep_rank is the most rows the caller will keep: the sweeps stop once only
 // rows that cannot be among them are still rotating (keep_rank >= rows
-// disables this).
+// disables this).  act (device, may be NULL) restricts the sweeps to the rows
+// act[1..act[0]], all other pairs being orthogonal already.
 cudaError_t jacobi_rows(cplx* A, int rows, int len, int max_sweeps, double tol,
                         const double* anorm2, double skip_rel, int keep_rank,
                         unsigned int* dev_state, int* stamps, double* wts, double* nref,
-                        cudaStream_t st);
+                        const int* act, cudaStream_t st);
 // Several jacobi_rows problems in one cooperative launch (the truncated
 // splits of concurrent evolutions).  Each item is one matrix with its own
 // dev_state, stamps, wts and nref as jacobi_rows takes them, cleared
@@ -239,6 +274,7 @@ struct JacobiItem {
   double* nref;
   double tol, skip_rel;
   int rows, len, max_sweeps, keep_rank;
+  const int* act;
 };
 constexpr int kJacobiGroupMax = 32;
 struct JacobiGroup {

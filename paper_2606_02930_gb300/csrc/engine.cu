@@ -45,6 +45,12 @@ constexpr double kEps = 2.220446049250313e-16;
 constexpr int kJacobiSweeps = 30;
 constexpr int kMaxKrylov = 32;
 constexpr double kEmuMinWork = 2.0e6;    // complex MACs below which GEMMs stay native
+// Rows from which the Jacobi of a split is preconditioned.  A whole split of k x k,
+// without and with it: k = 16 0.81 and 0.70 ms, 24 1.36 and 0.91, 32 2.00 and
+// 1.05, 64 4.36 and 2.05, 128 9.14 and 3.48, 512 69.7 and 22.6.  Below 16 rows
+// one cluster step covers the whole matrix and the GEMMs' launches outweigh the
+// few rounds saved.
+constexpr int kPreMinRows = 16;
 // Algorithmic FP64 work of a truncated SVD of a p x q complex block, as the
 // reference count that roofline figures divide by: the 22 n^3-class estimate
 // of 8.7 GFLOP for a 512 x 512 block, scaled by p q min(p, q).
@@ -64,7 +70,7 @@ struct HostRead {
   int counter;
   int pad;
   int lq_err;
-  int pad2;
+  int pre_err;
   unsigned int pairs[2];
   double disc;
   double res;
@@ -268,21 +274,26 @@ ite_status kernel_finish(ite_ctx ctx) {
 }
 
 // ------------------------------------------------------------------ contractions
+// large contractions on the tensor cores when the step asks for it; small
+// ones (edge bonds) stay on the FP64 pipe where launch latency dominates
+bool emulated(ite_ctx ctx, int M, int N, int K) {
+  return ctx->gemm_mode == 1 && (double)M * N * K >= kEmuMinWork && K >= 16;
+}
+
 // Plain GEMM helpers.  Row-major matrices; strides in complex units.
 ite_status gemm(ite_ctx ctx, int M, int N, int K, const cplx* A, long long sAm, long long sAk,
                 bool conjA, const cplx* B, long long sBk, long long sBn, bool conjB, cplx* Cm,
                 long long ldc, cplx alpha = C(1), cplx beta = C(0), const cplx* Z = nullptr,
                 cplx gamma = C(0), int batch = 1, long long sAb = 0, long long sBb = 0,
-                long long sCb = 0) {
+                long long sCb = 0, const int* run_if = nullptr) {
   GemmArgs g;
+  g.run_if = run_if;
   g.M = M; g.N = N; g.K = K; g.batch = batch;
   g.A = A; g.sAm = sAm; g.sAk = sAk; g.sAb = sAb; g.conjA = conjA;
   g.B = B; g.sBk = sBk; g.sBn = sBn; g.sBb = sBb; g.conjB = conjB;
   g.C = Cm; g.ldc = ldc; g.sCb = sCb;
   g.alpha = alpha; g.beta = beta; g.Z = Z; g.gamma = gamma;
-  // large contractions on the tensor cores when the step asks for it; small
-  // ones (edge bonds) stay on the FP64 pipe where launch latency dominates
-  if (ctx->gemm_mode == 1 && (double)M * N * K >= kEmuMinWork && K >= 16) {
+  if (emulated(ctx, M, N, K)) {
     CS(buf_ensure(ctx, ctx->ws_emu, zgemm_emu_scratch_bytes(M, N, K)));
     CK(zgemm_emu(g, ctx->ws_emu.p, ctx->ws_emu.n, reinterpret_cast<int*>(ctx->dcounter) + 10,
                  ctx->stream));
@@ -444,6 +455,58 @@ ite_status merge(ite_ctx ctx, int d, int chl, int chm, int chr, const cplx* K1, 
               (long long)d * chr);
 }
 
+// Y += D Y (D k x k, Y k x len) unless *run_if is 0; tmp holds k x len.  The
+// emulated GEMM reads Y only while slicing it, so it works in place.
+ite_status add_left(ite_ctx ctx, const cplx* D, cplx* Y, int k, int len, cplx* tmp,
+                    const int* run_if) {
+  if (emulated(ctx, k, len, k))
+    return gemm(ctx, k, len, k, D, k, 1, false, Y, len, 1, false, Y, len, C(1), C(1), nullptr, C(0),
+                1, 0, 0, 0, run_if);
+  CS(gemm(ctx, k, len, k, D, k, 1, false, Y, len, 1, false, tmp, len, C(1), C(0), Y, C(1), 1, 0, 0,
+          0, run_if));
+  CK(vec_copy_if(Y, tmp, (long long)k * len, run_if, true, ctx->stream));
+  return ITE_OK;
+}
+
+// S (k x p) = U R with U unitary and the rows of S orthogonal up to what act
+// lists (svd_pre.cu has the method); R is scratch afterwards.  Its matrices lie
+// in the Krylov basis' workspace, which no split needs.
+ite_status precondition(ite_ctx ctx, cplx* R, cplx* S, int k, int p, const double* anorm2,
+                        double skip_rel, double tol, const int** act, const int** err) {
+  CS(buf_ensure(ctx, ctx->ws_V, svd_pre_bytes(k, p)));
+  const SvdPre s = svd_pre_carve(ctx->ws_V.p, k, p);
+  cplx *A = s.K[0], *B = s.K[1], *W = s.K[2], *W2 = s.K[3];
+  auto gram = [&](const cplx* Y, int len, cplx* G, const int* run_if = nullptr) {
+    return gemm(ctx, k, k, len, Y, len, 1, false, Y, 1, len, true, G, k, C(1), C(0), nullptr, C(0),
+                1, 0, 0, 0, run_if);
+  };
+  CK(svd_pre_rotate(s, R, k, p, anorm2, ctx->stream));
+  for (int it = 0; it < 3; ++it) {
+    const int* on = it == 0 ? nullptr : it == 1 ? s.ok : s.gate_n;
+    CS(gram(A, k, B, on));
+    CK(svd_pre_orth(s, B, k, it, ctx->stream));
+    CS(add_left(ctx, B, A, k, k, W, it == 0 ? s.ok : on));
+  }
+  CS(gemm(ctx, k, p, k, A, k, 1, false, R, p, 1, false, S, p, C(1), C(0), nullptr, C(0), 1, 0, 0, 0,
+          s.ok));
+  CK(vec_copy_if(S, R, (long long)k * p, s.ok, false, ctx->stream));
+  for (int it = 0; it < 2; ++it) {
+    CS(gram(S, p, B));
+    CK(svd_pre_corr(s, B, k, tol, anorm2, skip_rel, A, ctx->stream));
+    CS(gemm(ctx, k, k, k, A, k, 1, false, A, k, 1, false, W, k, C(1), C(0), nullptr, C(0), 1, 0, 0,
+            0, s.gate_w));
+    CS(gemm(ctx, k, k, k, W, k, 1, false, W, k, 1, false, W2, k, C(1), C(0), nullptr, C(0), 1, 0, 0,
+            0, s.gate_w2));
+    CK(svd_pre_comb(s, A, W, W2, k, ctx->stream));
+    CS(add_left(ctx, A, S, k, p, R, s.gate));
+  }
+  CS(gram(S, p, B));
+  CK(svd_pre_list(s, B, k, tol, anorm2, skip_rel, ctx->stream));
+  *act = s.act;
+  *err = s.err;
+  return ITE_OK;
+}
+
 // Truncated SVD of X (m x n) into left (m x r) and right (r x n); returns r.
 // The rows of Xr are indexed by the side whose isometry is wanted: Xr = X
 // when centre_right (left = U_r), Xr = X^H otherwise (right = V_r^H).  The
@@ -487,26 +550,34 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
     CK(svd_lq(W, p, q, beta, nullptr, lqstate, ctx->stream));
   }
   CK(svd_lq_r(W, beta, p, q, R, ctx->stream));
-  // 3. one-sided Jacobi on the k rows (length p) of R
+  // 3. one-sided Jacobi on the k rows (length p) of R, preconditioned where
+  // its rounds outweigh the GEMMs of the preconditioner
+  cplx* D = R;          // Sigma U^H in the end; the other of R and W is free
+  const int* act = nullptr;
+  const int* pre_err = nullptr;
   {
     Scope jacobi_scope(ctx, P_JACOBI);
     const double tol = std::max(1e-15, p * kEps);
+    if (k >= kPreMinRows) {
+      D = W;
+      CS(precondition(ctx, R, D, k, p, anorm2, skip_weight(cutoff), tol, &act, &pre_err));
+    }
     if (ctx->group && k >= 3) {
       // the same Jacobi, launched together with other contexts' splits
       CK(jacobi_prepare(k, jstate, stamps, ctx->stream));
-      const JacobiItem item{R, anorm2, jstate, stamps, wts, nref, tol, skip_weight(cutoff),
-                            k, p, kJacobiSweeps, chi_max};
+      const JacobiItem item{D, anorm2, jstate, stamps, wts, nref, tol, skip_weight(cutoff),
+                            k, p, kJacobiSweeps, chi_max, act};
       CK(group_jacobi(ctx->group, item, ctx->group_ready, ctx->group_done, ctx->group_state,
                       ctx->stream));
     } else {
-      CK(jacobi_rows(R, k, p, kJacobiSweeps, tol, anorm2, skip_weight(cutoff), chi_max, jstate,
-                     stamps, wts, nref, ctx->stream));
+      CK(jacobi_rows(D, k, p, kJacobiSweeps, tol, anorm2, skip_weight(cutoff), chi_max, jstate,
+                     stamps, wts, nref, act, ctx->stream));
     }
   }
   // 4. singular values, order and rank
   int* rank_dev = reinterpret_cast<int*>(ctx->dscal + 6);
   double* disc_dev = ctx->dscal + 7;
-  CK(svd_rank(R, k, p, sigma, perm, sorted, chi_max, cutoff, kWeightFloor, kTieRel, rank_dev,
+  CK(svd_rank(D, k, p, sigma, perm, sorted, chi_max, cutoff, kWeightFloor, kTieRel, rank_dev,
               disc_dev, ctx->stream));
   CK(cudaMemcpyAsync(&ctx->hr->rank, rank_dev, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaMemcpyAsync(&ctx->hr->disc, disc_dev, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
@@ -517,8 +588,11 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
                      ctx->stream));
   CK(cudaMemcpyAsync(&ctx->hr->steps, reinterpret_cast<int*>(ctx->dcounter) + 10, sizeof(int),
                      cudaMemcpyDeviceToHost, ctx->stream));
+  ctx->hr->pre_err = 0;
+  if (pre_err)
+    CK(cudaMemcpyAsync(&ctx->hr->pre_err, pre_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CS(sync(ctx));
-  if (ctx->hr->counter != 0 || ctx->hr->lq_err != 0)
+  if (ctx->hr->counter != 0 || ctx->hr->lq_err != 0 || ctx->hr->pre_err != 0)
     return fail(ctx, ITE_ETIMEOUT, "SVD grid barrier wait ran out");
   if (ctx->hr->steps != 0) return fail(ctx, ITE_ETIMEOUT, "tensor-core GEMM wait ran out");
   ctx->jacobi_sweeps_total += ctx->hr->pad;
@@ -536,11 +610,11 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
     CK(cudaMemsetAsync(sigma_out, 0, sizeof(double) * std::min(m, n), ctx->stream));
     CK(cudaMemcpyAsync(sigma_out, sorted, sizeof(double) * k, cudaMemcpyDeviceToDevice, ctx->stream));
   }
-  // 5. factors: Uh = U_r^H (r x p) in the LQ workspace (free again), then
+  // 5. factors: Uh = U_r^H (r x p) in the workspace that is free, then
   // the projection.  X is read in full before the isometry side is written,
   // so X may share memory with that side (the gauge moves do).
-  cplx* Uh = W;
-  CK(svd_gather_uh(R, p, perm, sorted, r, Uh, ctx->stream));
+  cplx* Uh = D == R ? W : R;
+  CK(svd_gather_uh(D, p, perm, sorted, r, Uh, ctx->stream));
   if (!centre_right) {
     // left = X V_r (m x r), right = V_r^H (r x n)
     CS(gemm(ctx, m, r, n, X, n, 1, false, Uh, 1, n, true, left, r));

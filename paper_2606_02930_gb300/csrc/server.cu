@@ -103,7 +103,8 @@ size_t estimate_bytes(const ite_job* j) {
   // the MPS and its three work copies, left/right environments of x and of
   // the right-hand side, Krylov basis, two contraction intermediates and the
   // sweep's other two-site buffers
-  long long elems = 4 * mps + 2 * envs + 2 * ovs + (long long)(krylov + 1) * nmax +
+  // (the basis' room also holds the splits' preconditioner, up to 6 nmax)
+  long long elems = 4 * mps + 2 * envs + 2 * ovs + (long long)std::max(krylov + 1, 6) * nmax +
                     2LL * D * nmax + 6 * nmax;
   // Gauss-Legendre: q more MPS copies and overlap environments per fit target
   const int q = j->scheme == ITE_GAUSS_LEGENDRE_2 ? 2

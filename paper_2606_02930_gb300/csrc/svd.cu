@@ -638,11 +638,16 @@ k_jacobi_round(cplx* A, int len, double tol, const double* anorm2, double skip_r
 // left the pair orthogonal), examining it again cannot fire and is skipped.
 constexpr double kKeepMargin = 1e-2;
 __global__ void __launch_bounds__(TPP)
-k_jacobi_persistent(cplx* A, int rows, int len, int pp, double tol, const double* anorm2,
+k_jacobi_persistent(cplx* A, int rows, int len, double tol, const double* anorm2,
                     double skip_rel, int max_sweeps, int keep_rank, unsigned int* st, int* stamps,
-                    double* wts, double* nref) {
-  const unsigned int nb = gridDim.x;
+                    double* wts, double* nref, const int* act) {
+  unsigned int nb = gridDim.x;
   const int tid = threadIdx.x;
+  // the rows that take part, and their number made even (at least two rounds a
+  // sweep, for the reset of the counters)
+  const int nrow = act ? act[0] : rows;
+  if (nrow < 2) return;
+  const int pp = max(4, nrow + (nrow & 1));
   const double skip = skip_rel * (anorm2 ? *anorm2 : 0.0);
   int* counters = reinterpret_cast<int*>(st + S_CNT);
   unsigned long long* maxws = reinterpret_cast<unsigned long long*>(st + S_MAXW);
@@ -650,6 +655,8 @@ k_jacobi_persistent(cplx* A, int rows, int len, int pp, double tol, const double
   // the tracked squared norms start from the rows themselves
   team_row_norms(A, len, blockIdx.x, rows, (int)nb, wts, nref);
   if (!grid_barrier(st, nb)) return;
+  if ((int)nb > pp / 2) nb = pp / 2;       // blocks without a pair leave
+  if (blockIdx.x >= nb) return;
   for (int sw = 0; sw < max_sweeps; ++sw) {
     int* cnt = counters + (sw & 1);
     unsigned long long* maxw = maxws + (sw & 1);
@@ -661,8 +668,12 @@ k_jacobi_persistent(cplx* A, int rows, int len, int pp, double tol, const double
       const int g = sw * (pp - 1) + r;
       for (int k = blockIdx.x; k < pp / 2; k += (int)nb) {
         int u = player(k, r, pp), v = player(pp - 1 - k, r, pp);
-        if (u >= rows || v >= rows) continue;
+        if (u >= nrow || v >= nrow) continue;
         if (u > v) { const int t = u; u = v; v = t; }
+        if (act) {
+          u = act[1 + u];
+          v = act[1 + v];
+        }
         // from the second sweep on, a pair neither of whose rows has been
         // rotated since it was last examined is skipped
         bool skipped;
@@ -724,10 +735,13 @@ k_jacobi_grouped(const __grid_constant__ JacobiGroup g, unsigned int* gst) {
   __shared__ unsigned int s_ex[kJacobiGroupMax], s_rot[kJacobiGroupMax];
   __shared__ int s_done[kJacobiGroupMax], s_act[kJacobiGroupMax];
   __shared__ double s_skip[kJacobiGroupMax];
+  __shared__ int s_rows[kJacobiGroupMax], s_pp[kJacobiGroupMax];   // rows that take part
   const int n = g.n;
   for (int j = tid; j < n; j += TPP) {
     s_ex[j] = s_rot[j] = 0u;
-    s_done[j] = 0;
+    s_rows[j] = g.it[j].act ? g.it[j].act[0] : g.it[j].rows;
+    s_pp[j] = max(4, s_rows[j] + (s_rows[j] & 1));
+    s_done[j] = s_rows[j] < 2;
     s_skip[j] = g.it[j].skip_rel * (g.it[j].anorm2 ? *g.it[j].anorm2 : 0.0);
   }
   __syncthreads();
@@ -744,7 +758,7 @@ k_jacobi_grouped(const __grid_constant__ JacobiGroup g, unsigned int* gst) {
     // matrices still sweeping (every block decides alike)
     int total = 0;
     for (int j = 0; j < n; ++j) {
-      const int pp = g.it[j].rows + (g.it[j].rows & 1);
+      const int pp = s_pp[j];
       const bool act = !s_done[j] && G / (pp - 1) < g.it[j].max_sweeps;
       if (tid == 0) s_act[j] = act;
       if (act) total += pp / 2;
@@ -752,7 +766,7 @@ k_jacobi_grouped(const __grid_constant__ JacobiGroup g, unsigned int* gst) {
     if (total == 0) break;
     if (blockIdx.x == 0 && tid == 0) {
       for (int j = 0; j < n; ++j) {
-        const int pp = g.it[j].rows + (g.it[j].rows & 1);
+        const int pp = s_pp[j];
         const int sw = G / (pp - 1);
         if (s_act[j] && G % (pp - 1) == 1) {
           reinterpret_cast<int*>(g.it[j].st + S_CNT)[(sw + 1) & 1] = 0;
@@ -765,16 +779,20 @@ k_jacobi_grouped(const __grid_constant__ JacobiGroup g, unsigned int* gst) {
       int j = 0, k = f;
       for (;; ++j) {
         if (!s_act[j]) continue;
-        const int half = (g.it[j].rows + (g.it[j].rows & 1)) / 2;
+        const int half = s_pp[j] / 2;
         if (k < half) break;
         k -= half;
       }
       const JacobiItem& it = g.it[j];
-      const int rows = it.rows, pp = rows + (rows & 1);
+      const int nrow = s_rows[j], pp = s_pp[j];
       const int sw = G / (pp - 1), r = G % (pp - 1);
       int u = player(k, r, pp), v = player(pp - 1 - k, r, pp);
-      if (u >= rows || v >= rows) continue;
+      if (u >= nrow || v >= nrow) continue;
       if (u > v) { const int t = u; u = v; v = t; }
+      if (it.act) {
+        u = it.act[1 + u];
+        v = it.act[1 + v];
+      }
       bool skipped;
       const PairOut o = jacobi_pair(it.A, it.len, u, v, it.tol, s_skip[j], it.wts, it.nref,
                                     it.stamps, sw > 0 ? G - (pp - 1) : -1, &skipped);
@@ -799,7 +817,7 @@ k_jacobi_grouped(const __grid_constant__ JacobiGroup g, unsigned int* gst) {
     for (int j = 0; j < n; ++j) {
       if (!s_act[j]) continue;
       const JacobiItem& it = g.it[j];
-      const int rows = it.rows, pp = rows + (rows & 1);
+      const int rows = it.rows, pp = s_pp[j];
       if (G % (pp - 1) != pp - 2) continue;
       const int sw = G / (pp - 1);
       if (blockIdx.x == 0 && tid == 0) it.st[S_SWEEPS] = (unsigned int)(sw + 1);
@@ -1055,7 +1073,7 @@ cudaError_t svd_lq_r(const cplx* W, const cplx* beta, int p, int q, cplx* R, cud
 cudaError_t jacobi_rows(cplx* A, int rows, int len, int max_sweeps, double tol,
                         const double* anorm2, double skip_rel, int keep_rank,
                         unsigned int* dev_state, int* stamps, double* wts, double* nref,
-                        cudaStream_t st) {
+                        const int* act, cudaStream_t st) {
   cudaError_t err = cudaMemsetAsync(dev_state, 0, S_WORDS * sizeof(unsigned int), st);
   if (err != cudaSuccess) return err;
   if (rows < 2) return cudaSuccess;
@@ -1075,8 +1093,8 @@ cudaError_t jacobi_rows(cplx* A, int rows, int len, int max_sweeps, double tol,
   if (err != cudaSuccess) return err;
   int nblk = pp / 2;
   if (nblk > max_blocks) nblk = max_blocks;
-  void* args[] = {&A, &rows, &len, (void*)&pp, &tol, &anorm2, &skip_rel, &max_sweeps, &keep_rank,
-                  &dev_state, &stamps, &wts, &nref};
+  void* args[] = {&A, &rows, &len, &tol, &anorm2, &skip_rel, &max_sweeps, &keep_rank,
+                  &dev_state, &stamps, &wts, &nref, &act};
   count_launches(1);
   return cudaLaunchCooperativeKernel((void*)k_jacobi_persistent, dim3(nblk), dim3(TPP), args, 0,
                                      st);

@@ -1,0 +1,751 @@
+// Preconditioner of the one-sided Jacobi of the truncated splits.
+//
+// The FP64 Jacobi (svd.cu) is a chain of one grid barrier per round and of
+// FP64 work on a pipe that issues two DFMA per clock and SM: 512 rows take 11
+// sweeps of 511 rounds of about 10 us.  Nearly all of that work only brings
+// rows that start far from orthogonal to a few digits of orthogonality, which
+// does not need FP64.  So the split first rotates the rows of R (k x p) by a
+// unitary V found in fp32, V R with rows orthogonal to about 1e-6:
+//   1. k_jacobi32: one-sided block Jacobi in fp32 on the rows of [R | I], one
+//      block pair (32 rows) per thread-block cluster and step, whose Gram
+//      matrix is diagonalised by Jacobi rotations in shared memory;
+//   2. V is made unitary to FP64 rounding by two or three Newton-Schulz steps
+//      V <- V - (V V^H - I) V / 2, and applied, S = V R, in FP64 (FP64-class)
+//      GEMMs: S^H S = R^H R to rounding, whatever the quality of V;
+//   3. twice, the Gram matrix G = S S^H gives the first-order rotations
+//      E_ij = t e^{i theta} of every pair that is not yet orthogonal (the
+//      Jacobi rotation's tangent, kept only where it is small), and
+//      S <- S + (E + E^2/2 - E^4/8) S, unitary to E^6: quadratic convergence
+//      for well separated rows;
+//   4. a last Gram matrix lists the rows that still have a pair above the
+//      Jacobi's tolerance (members of near-degenerate groups, or all rows if
+//      a check below failed); the FP64 Jacobi runs on those rows only.
+// Every transformation applied is unitary to FP64 rounding, and the FP64
+// Jacobi's criterion decides what remains, so the factors are as accurate as
+// without the preconditioner.  S is updated by small corrections D S rather
+// than replaced by Q S so that the light rows keep their relative accuracy:
+// the FP64-class GEMM's error is relative to the largest entry of D's row.
+// Guards: V is dropped (S = R, all rows go to the Jacobi) unless
+// |V V^H - I|_inf < 1e-2, from which three Newton-Schulz steps reach rounding;
+// a correction is dropped unless |E|_inf <= 2e-3.
+#include <cooperative_groups.h>
+
+#include <mutex>
+
+#include "common.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace ite {
+namespace {
+
+// control words (PreCtl in device memory, cleared before each use)
+constexpr int C_ARRIVE = 0, C_GEN = 1, C_ERR = 4, C_SWEEPS = 5;
+constexpr int C_OK = 8, C_GE = 9, C_GW = 10, C_GW2 = 11, C_COUNT = 12, C_GN = 13;
+constexpr int C_DELTA = 16, C_NU = 18;        // 64-bit words
+constexpr int C_OFF = 24;                     // per-sweep largest overlap (float bits)
+constexpr int C_WORDS = 64;
+constexpr int kSweeps32 = 16;
+static_assert(C_OFF + kSweeps32 <= C_WORDS, "control words");
+
+constexpr int PB = 16;                        // rows of a block
+constexpr int PM = 2 * PB;                    // rows of a block pair
+constexpr int PT = 256;                       // threads per CTA
+constexpr int GLD = PM + 1;                   // padded row of the Gram matrix
+constexpr int QLD = PM + 2;                   // padded row of Q^T (16-byte aligned pairs)
+constexpr float kStop32 = 1e-3f;              // largest overlap of the last sweep (its square remains)
+constexpr float kRot32 = 2e-7f;               // overlaps below this are fp32 rounding
+constexpr float kTiny32 = 1e-34f;             // squared norms below this (of 1) are left alone
+
+struct Pre32 {
+  float2* R;                                  // kp x pp, the scaled rows
+  float2* V;                                  // kp x kp, the accumulated rotation
+  int k, kp, pp, nb;                          // rows, padded rows, padded length, blocks
+  int pc, vc, chunk;                          // columns of R and V per CTA, columns staged at once
+};
+
+// Barrier over the clusters' first CTAs; bounded like grid_barrier (svd.cu).
+__device__ bool leader_barrier(unsigned int* st, unsigned int n) {
+  volatile unsigned int* gen = st + C_GEN;
+  const unsigned int g = *gen;
+  __threadfence();
+  if (atomicAdd(st + C_ARRIVE, 1u) == n - 1) {
+    atomicExch(st + C_ARRIVE, 0u);
+    __threadfence();
+    atomicAdd(st + C_GEN, 1u);
+  } else {
+    unsigned long long spins = 0;
+    while (*gen == g) {
+      if (*((volatile unsigned int*)(st + C_ERR)) != 0u) break;
+      if (++spins > (1ull << 24)) {
+        atomicExch(st + C_ERR, 1u);
+        break;
+      }
+      __nanosleep(20);
+    }
+  }
+  __threadfence();
+  return *((volatile unsigned int*)(st + C_ERR)) == 0u;
+}
+
+__device__ __forceinline__ int seat(int pos, int round, int n) {
+  return pos == 0 ? 0 : ((pos - 1 + round) % (n - 1)) + 1;
+}
+
+// Local column c of this CTA in the concatenated row [R | V] (two columns at
+// a time: pc and vc are even).
+__device__ __forceinline__ float4* col_ptr(const Pre32& a, int row, int rank, int c) {
+  float2* p = c < a.pc ? a.R + (long long)row * a.pp + (long long)rank * a.pc + c
+                       : a.V + (long long)row * a.kp + (long long)rank * a.vc + (c - a.pc);
+  return reinterpret_cast<float4*>(p);
+}
+
+// One cluster per block pair, the columns of the pair's rows dealt to its
+// CTAs.  Per step: each CTA stages its columns, forms its share of the 32 x 32
+// Gram matrix, the shares are added through distributed shared memory in a
+// fixed order, every CTA diagonalises the sum the same way and applies the
+// result to its own columns.
+// Bound: latency.  A step of the k = 512 case moves 8 MB through L2 and does
+// 50 MFLOP on 128 SMs (2 us); the 31 dependent rounds of the 32 x 32
+// diagonalisation take most of the rest.  16-row blocks: 8-row ones need
+// twice the steps and barriers for the same number of rounds, 32-row ones
+// leave half the SMs without a pair.  Whole 512 x 512 split (chi_max 256, cutoff
+// 1e-10): 69.3 ms with the FP64 Jacobi alone, 22.6 ms with the preconditioner
+// (none of the FP64 sweeps is left); 1024 x 1024: 324 ms and 79 ms.
+__global__ void __launch_bounds__(PT)
+k_jacobi32(Pre32 a, unsigned int* st) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int ncl = gridDim.x / C, cid = blockIdx.x / C;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  extern __shared__ float4 dyn[];
+  float2* part = reinterpret_cast<float2*>(dyn);            // PM x GLD
+  float2* G = part + PM * GLD;                              // PM x GLD
+  float2* QT = G + PM * GLD;                                // PM x QLD: QT[c][r] = Q[r][c]
+  float2* S = QT + PM * QLD;                                // PM x ld
+  __shared__ float4 rot[PB];
+  __shared__ int s_pos[PM];
+  __shared__ int s_off, s_ok;
+  const int lc = a.pc + a.vc, ld = a.chunk + 2;
+  const bool resident = lc <= a.chunk;
+  const int ty = tid >> 4, tx = tid & 15;
+
+  // rows of the pair (u, v): 0..15 of block u, then 0..15 of block v
+  auto stage = [&](int u, int v, int c0, int n) {
+    const int n2 = n >> 1;
+    for (int e = tid; e < PM * n2; e += PT) {
+      const int r = e / n2, c = 2 * (e - r * n2);
+      const int row = (r < PB ? u * PB + r : v * PB + r - PB);
+      *reinterpret_cast<float4*>(S + r * ld + c) = __ldcg(col_ptr(a, row, rank, c0 + c));
+    }
+  };
+
+  for (int sw = 0; sw < kSweeps32; ++sw) {
+    bool ok = true;
+    for (int rd = 0; rd < a.nb - 1; ++rd) {
+      for (int k = cid; k < a.nb / 2; k += ncl) {
+        int u = seat(k, rd, a.nb), v = seat(a.nb - 1 - k, rd, a.nb);
+        if (u > v) { const int t = u; u = v; v = t; }
+        // ---- share of the Gram matrix: thread (ty, tx) rows ty, ty+16 by tx, tx+16
+        float2 acc[2][2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) acc[i][j] = make_float2(0.f, 0.f);
+        for (int c0 = 0; c0 < (resident ? 1 : a.pc); c0 += a.chunk) {
+          const int n = resident ? lc : min(a.chunk, a.pc - c0);
+          const int ng = resident ? a.pc : n;
+          stage(u, v, c0, n);
+          __syncthreads();
+          for (int c = 0; c < ng; c += 2) {
+            float4 x[2], y[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              x[i] = *reinterpret_cast<const float4*>(S + (ty + PB * i) * ld + c);
+              y[i] = *reinterpret_cast<const float4*>(S + (tx + PB * i) * ld + c);
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+              for (int j = 0; j < 2; ++j) {
+                // x conj(y)
+                acc[i][j].x = fmaf(x[i].x, y[j].x, fmaf(x[i].y, y[j].y, acc[i][j].x));
+                acc[i][j].y = fmaf(x[i].y, y[j].x, fmaf(-x[i].x, y[j].y, acc[i][j].y));
+                acc[i][j].x = fmaf(x[i].z, y[j].z, fmaf(x[i].w, y[j].w, acc[i][j].x));
+                acc[i][j].y = fmaf(x[i].w, y[j].z, fmaf(-x[i].z, y[j].w, acc[i][j].y));
+              }
+          }
+          if (!resident) __syncthreads();
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) part[(ty + PB * i) * GLD + tx + PB * j] = acc[i][j];
+        cl.sync();
+        // ---- sum of the shares (upper triangle, mirrored); Q = I
+        for (int e = tid; e < PM * PM; e += PT) {
+          const int i = e / PM, j = e - i * PM;
+          if (i <= j) {
+            float2 s = make_float2(0.f, 0.f);
+            for (int r = 0; r < C; ++r) {
+              const float2 t = cl.map_shared_rank(part, r)[i * GLD + j];
+              s.x += t.x;
+              s.y += t.y;
+            }
+            if (i == j) {
+              // padding rows sort last and never rotate
+              const int row = i < PB ? u * PB + i : v * PB + i - PB;
+              G[i * GLD + i] = make_float2(row < a.k ? s.x : -1.f, 0.f);
+            } else {
+              G[i * GLD + j] = s;
+              G[j * GLD + i] = make_float2(s.x, -s.y);
+            }
+          }
+          QT[i * QLD + j] = make_float2(i == j ? 1.f : 0.f, 0.f);
+        }
+        if (tid == 0) s_off = 0;
+        __syncthreads();
+        // ---- one cyclic sweep of rotations: thread t < 16 forms those of the round
+        float off = 0.f;
+        for (int r = 0; r < PM - 1; ++r) {
+          if (tid < PB) {
+            int i = seat(tid, r, PM), j = seat(PM - 1 - tid, r, PM);
+            if (i > j) { const int t = i; i = j; j = t; }
+            const float al = G[i * GLD + i].x, be = G[j * GLD + j].x;
+            const float2 g = G[i * GLD + j];
+            float c = 1.f, sx = 0.f, sy = 0.f, tg = 0.f;
+            if (al > kTiny32 && be > kTiny32) {
+              // the overlap (hx, hy) = g / (|x| |y|): its square stays in range
+              // for rows of any weight
+              const float ra = rsqrtf(al), rb = rsqrtf(be);
+              const float hx = g.x * ra * rb, hy = g.y * ra * rb;
+              const float h2 = fmaf(hx, hx, hy * hy);
+              if (h2 > kRot32 * kRot32) {
+                const float ih = rsqrtf(h2), h = h2 * ih;
+                off = fmaxf(off, h);
+                // tangent of the rotation that zeroes g, |t| <= 1
+                const float ga = h * (al * ra) * (be * rb);
+                const float D = be - al, z = fabsf(D) / (2.f * ga);
+                const float t = 1.f / (z + sqrtf(fmaf(z, z, 1.f)));
+                const float q = fmaf(t, t, 1.f);
+                c = rsqrtf(q);
+                c = c * fmaf(-0.5f * q * c, c, 1.5f);
+                const float sg = (D >= 0.f ? c * t : -c * t) * ih;
+                sx = sg * hx;
+                sy = sg * hy;
+                tg = D >= 0.f ? t * ga : -t * ga;
+              }
+            }
+            rot[tid] = make_float4(c, sx, sy, tg);
+          }
+          __syncthreads();
+          {
+            // thread (ty, tx): the 2 x 2 block of row pair ty and column pair tx
+            int i = seat(ty, r, PM), j = seat(PM - 1 - ty, r, PM);
+            if (i > j) { const int t = i; i = j; j = t; }
+            int m = seat(tx, r, PM), n = seat(PM - 1 - tx, r, PM);
+            if (m > n) { const int t = m; m = n; n = t; }
+            const float4 ra = rot[ty], rb = rot[tx];
+            if (ty == tx) {
+              if (ra.y != 0.f || ra.z != 0.f) {
+                G[i * GLD + i].x -= ra.w;
+                G[j * GLD + j].x += ra.w;
+                G[i * GLD + j] = G[j * GLD + i] = make_float2(0.f, 0.f);
+              }
+            } else {
+              const float2 b00 = G[i * GLD + m], b01 = G[i * GLD + n];
+              const float2 b10 = G[j * GLD + m], b11 = G[j * GLD + n];
+              // rows: x' = c x - s y, y' = conj(s) x + c y
+              float2 p00, p01, p10, p11;
+              p00.x = ra.x * b00.x - (ra.y * b10.x - ra.z * b10.y);
+              p00.y = ra.x * b00.y - (ra.y * b10.y + ra.z * b10.x);
+              p01.x = ra.x * b01.x - (ra.y * b11.x - ra.z * b11.y);
+              p01.y = ra.x * b01.y - (ra.y * b11.y + ra.z * b11.x);
+              p10.x = (ra.y * b00.x + ra.z * b00.y) + ra.x * b10.x;
+              p10.y = (ra.y * b00.y - ra.z * b00.x) + ra.x * b10.y;
+              p11.x = (ra.y * b01.x + ra.z * b01.y) + ra.x * b11.x;
+              p11.y = (ra.y * b01.y - ra.z * b01.x) + ra.x * b11.y;
+              // columns: x' = c x - conj(s) y, y' = s x + c y
+              float2 o;
+              o.x = rb.x * p00.x - (rb.y * p01.x + rb.z * p01.y);
+              o.y = rb.x * p00.y - (rb.y * p01.y - rb.z * p01.x);
+              G[i * GLD + m] = o;
+              o.x = (rb.y * p00.x - rb.z * p00.y) + rb.x * p01.x;
+              o.y = (rb.y * p00.y + rb.z * p00.x) + rb.x * p01.y;
+              G[i * GLD + n] = o;
+              o.x = rb.x * p10.x - (rb.y * p11.x + rb.z * p11.y);
+              o.y = rb.x * p10.y - (rb.y * p11.y - rb.z * p11.x);
+              G[j * GLD + m] = o;
+              o.x = (rb.y * p10.x - rb.z * p10.y) + rb.x * p11.x;
+              o.y = (rb.y * p10.y + rb.z * p10.x) + rb.x * p11.y;
+              G[j * GLD + n] = o;
+            }
+            // rows m, n of Q, columns ty and ty + 16
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              float2* q = QT + (ty + PB * h) * QLD;
+              const float2 x = q[m], y = q[n];
+              q[m] = make_float2(rb.x * x.x - (rb.y * y.x - rb.z * y.y),
+                                 rb.x * x.y - (rb.y * y.y + rb.z * y.x));
+              q[n] = make_float2((rb.y * x.x + rb.z * x.y) + rb.x * y.x,
+                                 (rb.y * x.y - rb.z * x.x) + rb.x * y.y);
+            }
+          }
+          __syncthreads();
+        }
+        if (tid < PB) atomicMax(&s_off, __float_as_int(off));
+        // ---- heavier rows first
+        if (tid < PM) {
+          const float di = G[tid * GLD + tid].x;
+          int pos = 0;
+          for (int j = 0; j < PM; ++j) {
+            const float dj = G[j * GLD + j].x;
+            pos += (dj > di) || (dj == di && j < tid);
+          }
+          s_pos[tid] = pos;
+        }
+        __syncthreads();
+        if (tid == 0 && rank == 0) atomicMax(st + C_OFF + sw, (unsigned int)s_off);
+        // ---- rows <- Q rows: warp w the rows 8 (w % 4).., 64 columns at a time
+        const int r0 = 8 * (warp & 3);
+        for (int c0 = 0; c0 < lc; c0 += a.chunk) {
+          const int n = min(a.chunk, lc - c0);
+          if (!resident) {
+            __syncthreads();
+            stage(u, v, c0, n);
+            __syncthreads();
+          }
+          for (int cb = (warp >> 2) * 64; cb < n; cb += 128) {
+            const int c = cb + 2 * lane;
+            const bool in = c < n;
+            const float2* sp = S + (in ? c : 0);
+            float2 o[8][2];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o[i][0] = o[i][1] = make_float2(0.f, 0.f);
+#pragma unroll 4
+            for (int m = 0; m < PM; ++m) {
+              const float4 s = *reinterpret_cast<const float4*>(sp + m * ld);
+              const float4* qp = reinterpret_cast<const float4*>(QT + m * QLD + r0);
+#pragma unroll
+              for (int i2 = 0; i2 < 4; ++i2) {
+                const float4 q = qp[i2];
+                float2* o0 = o[2 * i2];
+                float2* o1 = o[2 * i2 + 1];
+                o0[0].x = fmaf(q.x, s.x, fmaf(-q.y, s.y, o0[0].x));
+                o0[0].y = fmaf(q.x, s.y, fmaf(q.y, s.x, o0[0].y));
+                o0[1].x = fmaf(q.x, s.z, fmaf(-q.y, s.w, o0[1].x));
+                o0[1].y = fmaf(q.x, s.w, fmaf(q.y, s.z, o0[1].y));
+                o1[0].x = fmaf(q.z, s.x, fmaf(-q.w, s.y, o1[0].x));
+                o1[0].y = fmaf(q.z, s.y, fmaf(q.w, s.x, o1[0].y));
+                o1[1].x = fmaf(q.z, s.z, fmaf(-q.w, s.w, o1[1].x));
+                o1[1].y = fmaf(q.z, s.w, fmaf(q.w, s.z, o1[1].y));
+              }
+            }
+            if (in) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const int pos = s_pos[r0 + i];
+                const int row = pos < PB ? u * PB + pos : v * PB + pos - PB;
+                *col_ptr(a, row, rank, c0 + c) =
+                    make_float4(o[i][0].x, o[i][0].y, o[i][1].x, o[i][1].y);
+              }
+            }
+          }
+        }
+        // a further pair of this cluster overwrites part, read by the others
+        cl.sync();
+      }
+      cl.sync();
+      if (rank == 0 && tid == 0) s_ok = leader_barrier(st, (unsigned int)ncl) ? 1 : 0;
+      cl.sync();
+      ok = *cl.map_shared_rank(&s_ok, 0) != 0;
+      if (!ok) break;
+    }
+    if (!ok) break;
+    if (blockIdx.x == 0 && tid == 0) st[C_SWEEPS] = (unsigned int)(sw + 1);
+    if (__int_as_float((int)__ldcg(st + C_OFF + sw)) <= kStop32) break;
+  }
+  cl.sync();                    // s_ok of the first CTA stays readable until here
+}
+
+// R32 = R / |R|_F with zero padding, V = I
+__global__ void k_pre_init(const cplx* __restrict__ R, int p, const double* anorm2, Pre32 a) {
+  const double n2 = *anorm2;
+  const double s = n2 > 0.0 && isfinite(n2) ? rsqrt(n2) : 0.0;
+  const long long w = a.pp + a.kp, tot = w * a.kp;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
+       e += (long long)gridDim.x * blockDim.x) {
+    const int i = (int)(e / w), c = (int)(e - (long long)i * w);
+    if (c < a.pp) {
+      float2 v = make_float2(0.f, 0.f);
+      if (i < a.k && c < p) {
+        const cplx x = R[(long long)i * p + c];
+        v = make_float2((float)(x.x * s), (float)(x.y * s));
+      }
+      a.R[(long long)i * a.pp + c] = v;
+    } else {
+      a.V[(long long)i * a.kp + c - a.pp] = make_float2(i == c - a.pp ? 1.f : 0.f, 0.f);
+    }
+  }
+}
+
+__global__ void k_pre_export(Pre32 a, cplx* __restrict__ V) {
+  const long long tot = (long long)a.k * a.k;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
+       e += (long long)gridDim.x * blockDim.x) {
+    const int i = (int)(e / a.k), c = (int)(e - (long long)i * a.k);
+    const float2 v = a.V[(long long)i * a.kp + c];
+    V[e] = cmake(v.x, v.y);
+  }
+}
+
+constexpr int RT = 128;                       // threads of the row kernels
+
+__device__ __forceinline__ double block_sum(double v) {
+  __shared__ double sh[RT / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double s = 0.0;
+#pragma unroll
+  for (int w = 0; w < RT / 32; ++w) s += sh[w];
+  return s;
+}
+
+// The largest row sum over the blocks, in *word; the last block to finish
+// gets true (and sees every contribution).  Row sums are not negative, so
+// their bit patterns order like them, and a NaN is above them all.
+__device__ __forceinline__ bool max_over_blocks(double v, unsigned int* ctl, int word) {
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    atomicMax(reinterpret_cast<unsigned long long*>(ctl + word),
+              (unsigned long long)__double_as_longlong(v));
+    __threadfence();
+    last = atomicAdd(ctl + C_COUNT, 1u) == gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  return last;
+}
+
+constexpr double kDeltaMax = 1e-2;            // |V V^H - I|_inf of a usable V
+constexpr double kDeltaEnd = 1e-8;            // below this one more step is the last
+
+// M = V V^H becomes the Newton-Schulz correction -(M - I) / 2, which leaves
+// 3/4 |M - I|^2.  The first step decides whether V is usable (then three steps
+// reach rounding), the second whether a third is needed.
+__global__ void __launch_bounds__(RT) k_pre_orth(cplx* M, int k, unsigned int* ctl, int step) {
+  if (step > 0 && ctl[step == 1 ? C_OK : C_GN] == 0u) return;
+  const int i = blockIdx.x;
+  double s = 0.0;
+  for (int j = threadIdx.x; j < k; j += RT) {
+    cplx v = M[(long long)i * k + j];
+    if (j == i) v.x -= 1.0;
+    s += fabs(v.x) + fabs(v.y);
+    M[(long long)i * k + j] = cmake(-0.5 * v.x, -0.5 * v.y);
+  }
+  s = block_sum(s);
+  if (step > 1) return;
+  if (max_over_blocks(s, ctl, C_DELTA) && threadIdx.x == 0) {
+    unsigned long long* w = reinterpret_cast<unsigned long long*>(ctl + C_DELTA);
+    const double d = __longlong_as_double((long long)__ldcg(w));
+    if (step == 0) ctl[C_OK] = d < kDeltaMax && ctl[C_ERR] == 0u ? 1u : 0u;
+    else ctl[C_GN] = d > kDeltaEnd ? 1u : 0u;
+    ctl[C_COUNT] = 0u;
+    *w = 0ull;
+  }
+}
+
+__global__ void k_copy_if(cplx* y, const cplx* x, long long n, const unsigned int* flag, int want) {
+  if ((*flag != 0u) != (want != 0)) return;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
+       e += (long long)gridDim.x * blockDim.x)
+    y[e] = x[e];
+}
+
+constexpr double kPairTan = 2.5e-4;           // tangents above this are left to the Jacobi
+constexpr double kNuMax = 2e-3;
+
+// E from G = S S^H: E_ij = -sign(D) t g_ij / |g_ij| (D = G_jj - G_ii, t the tangent of
+// the rotation that makes the pair orthogonal), exactly anti-Hermitian because
+// both halves come from the upper triangle.  The last block sets the gates of
+// what follows from nu = |E|_inf: E^2 counts above 4e-9, E^4 above 1e-4.
+__global__ void __launch_bounds__(RT)
+k_pre_corr(const cplx* __restrict__ G, int k, double tol, const double* anorm2, double skip_rel,
+           cplx* __restrict__ E, unsigned int* ctl) {
+  const int i = blockIdx.x;
+  const double skip = skip_rel * *anorm2;
+  const double al = G[(long long)i * k + i].x;
+  double s = 0.0;
+  for (int j = threadIdx.x; j < k; j += RT) {
+    cplx e = cmake(0.0, 0.0);
+    if (j != i) {
+      const double be = G[(long long)j * k + j].x;
+      const cplx g = i < j ? G[(long long)i * k + j] : cconj(G[(long long)j * k + i]);
+      const double g2 = fma(g.x, g.x, g.y * g.y);
+      if (g2 > tol * tol * al * be && g2 > 0.0 && (al > skip || be > skip)) {
+        // (i < j) D and sign as the upper element has them
+        const double D = i < j ? be - al : al - be;
+        const double u = 2.0 / (fabs(D) + sqrt(fma(D, D, 4.0 * g2)));
+        if (u * u * g2 < kPairTan * kPairTan) {
+          const double c = (D >= 0.0) == (i < j) ? -u : u;
+          e = cmake(c * g.x, c * g.y);
+          s += u * sqrt(g2);
+        }
+      }
+    }
+    E[(long long)i * k + j] = e;
+  }
+  s = block_sum(s);
+  if (max_over_blocks(s, ctl, C_NU) && threadIdx.x == 0) {
+    unsigned long long* w = reinterpret_cast<unsigned long long*>(ctl + C_NU);
+    const double nu = __longlong_as_double((long long)__ldcg(w));
+    const bool on = nu > 0.0 && nu <= kNuMax;
+    ctl[C_GE] = on;
+    ctl[C_GW] = on && nu > 4e-9;
+    ctl[C_GW2] = on && nu > 1e-4;
+    ctl[C_COUNT] = 0u;
+    *w = 0ull;
+  }
+}
+
+// E <- E + W / 2 - W2 / 8 (W = E^2, W2 = E^4)
+__global__ void k_pre_comb(cplx* E, const cplx* W, const cplx* W2, long long n,
+                           const unsigned int* ctl) {
+  const bool w = ctl[C_GW] != 0u, w2 = ctl[C_GW2] != 0u;
+  if (!w) return;
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
+       e += (long long)gridDim.x * blockDim.x) {
+    cplx v = cadd(E[e], cscale(W[e], 0.5));
+    if (w2) v = cadd(v, cscale(W2[e], -0.125));
+    E[e] = v;
+  }
+}
+
+// flag[i] = 1 if row i belongs to a pair that is not orthogonal to tol.  For a
+// pair of which one row is below the skip weight (it can never be kept), what
+// counts is what its rotation would change in the heavier row, as in the
+// Jacobi's own stopping rule.  All rows if V was dropped.
+__global__ void __launch_bounds__(RT)
+k_pre_flag(const cplx* __restrict__ G, int k, double tol, const double* anorm2, double skip_rel,
+           int* flag, const unsigned int* ctl) {
+  const int i = blockIdx.x;
+  const double skip = skip_rel * *anorm2;
+  const double al = G[(long long)i * k + i].x;
+  int need = ctl[C_OK] == 0u;
+  for (int j = threadIdx.x; j < k; j += RT) {
+    if (j == i) continue;
+    const double be = G[(long long)j * k + j].x;
+    const cplx g = i < j ? G[(long long)i * k + j] : G[(long long)j * k + i];
+    const double g2 = fma(g.x, g.x, g.y * g.y);
+    if (al > skip && be > skip) {
+      if (g2 > tol * tol * al * be) need = 1;
+    } else if (al > skip || be > skip) {
+      const double D = be - al, lo = fmin(al, be), hi = fmax(al, be);
+      const double u = 2.0 / (fabs(D) + sqrt(fma(D, D, 4.0 * g2)));
+      if (g2 > 0.0 && u * u * g2 * lo > tol * tol * hi) need = 1;
+    }
+  }
+  need = __syncthreads_or(need);
+  if (threadIdx.x == 0) flag[i] = need;
+}
+
+// act[0] = number of flagged rows, act[1..] their indices in order (one block)
+__global__ void __launch_bounds__(1024) k_pre_compact(const int* flag, int k, int* act) {
+  __shared__ int wsum[32];
+  __shared__ int base;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (threadIdx.x == 0) base = 0;
+  __syncthreads();
+  for (int i0 = 0; i0 < k; i0 += 1024) {
+    const int i = i0 + threadIdx.x;
+    const bool f = i < k && flag[i] != 0;
+    const unsigned int m = __ballot_sync(0xffffffffu, f);
+    if (lane == 0) wsum[w] = __popc(m);
+    __syncthreads();
+    int before = base;
+    for (int x = 0; x < w; ++x) before += wsum[x];
+    if (f) act[1 + before + __popc(m & ((1u << lane) - 1u))] = i;
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int x = 0; x < 32; ++x) base += wsum[x];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) act[0] = base;
+}
+
+int grid_for(long long tot) {
+  long long g = (tot + 255) / 256;
+  return (int)(g > 1216 ? 1216 : g < 1 ? 1 : g);
+}
+
+long long round_up(long long x, long long m) { return (x + m - 1) / m * m; }
+
+struct PreDims {
+  int kp, pp;
+};
+PreDims pre_dims(int k, int p) { return {(int)round_up(k, PM), (int)round_up(p, 32)}; }
+
+constexpr size_t kFixedSmem = (size_t)PM * (2 * GLD + QLD) * sizeof(float2);
+constexpr int kChunkMax = 640;                // columns staged at once: 32 x 642 x 8 B = 164 KB
+
+// Clusters of C CTAs with this much shared memory that can be resident at
+// once on the current device, cached per (device, C, columns); several host
+// threads may ask at once.
+struct ClusterCapacity {
+  std::mutex mu;
+  struct Entry { int dev, C, chunk, n; };
+  Entry e[64];
+  int used = 0;
+} g_cap;
+
+void launch_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int grid, int C, size_t smem,
+                   cudaStream_t st, bool coop) {
+  *cfg = cudaLaunchConfig_t();
+  cfg->gridDim = dim3(grid);
+  cfg->blockDim = dim3(PT);
+  cfg->dynamicSmemBytes = smem;
+  cfg->stream = st;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeCooperative;
+  at[1].val.cooperative = 1;
+  cfg->attrs = at;
+  cfg->numAttrs = coop ? 2 : 1;
+}
+
+cudaError_t cluster_capacity(int C, int chunk, int* n) {
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  std::lock_guard<std::mutex> lock(g_cap.mu);
+  for (int i = 0; i < g_cap.used; ++i)
+    if (g_cap.e[i].dev == dev && g_cap.e[i].C == C && g_cap.e[i].chunk == chunk) {
+      *n = g_cap.e[i].n;
+      return cudaSuccess;
+    }
+  const size_t smem = kFixedSmem + (size_t)PM * (chunk + 2) * sizeof(float2);
+  err = cudaFuncSetAttribute(k_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(kFixedSmem + (size_t)PM * (kChunkMax + 2) * sizeof(float2)));
+  if (err != cudaSuccess) return err;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[2];
+  launch_config(&cfg, at, C * 1024, C, smem, nullptr, false);
+  err = cudaOccupancyMaxActiveClusters(n, k_jacobi32, &cfg);
+  if (err != cudaSuccess) return err;
+  if (g_cap.used < 64) g_cap.e[g_cap.used++] = {dev, C, chunk, *n};
+  return cudaSuccess;
+}
+
+}  // namespace
+
+size_t svd_pre_bytes(int k, int p) {
+  const PreDims d = pre_dims(k, p);
+  return (size_t)d.kp * (d.pp + d.kp) * sizeof(float2) + 4 * (size_t)k * k * sizeof(cplx) +
+         (size_t)(2 * k + 1) * sizeof(int) + C_WORDS * sizeof(int) + 6 * 256;
+}
+
+SvdPre svd_pre_carve(void* ws, int k, int p) {
+  const PreDims d = pre_dims(k, p);
+  char* c = static_cast<char*>(ws);
+  SvdPre s;
+  auto take = [&](size_t bytes) {
+    char* r = c;
+    c += round_up((long long)bytes, 256);
+    return r;
+  };
+  s.rows32 = take((size_t)d.kp * (d.pp + d.kp) * sizeof(float2));
+  for (cplx*& m : s.K) m = reinterpret_cast<cplx*>(take((size_t)k * k * sizeof(cplx)));
+  s.act = reinterpret_cast<int*>(take((size_t)(2 * k + 1) * sizeof(int)));
+  s.ctl = reinterpret_cast<unsigned int*>(take(C_WORDS * sizeof(int)));
+  s.ok = reinterpret_cast<int*>(s.ctl + C_OK);
+  s.gate_n = reinterpret_cast<int*>(s.ctl + C_GN);
+  s.gate = reinterpret_cast<int*>(s.ctl + C_GE);
+  s.gate_w = reinterpret_cast<int*>(s.ctl + C_GW);
+  s.gate_w2 = reinterpret_cast<int*>(s.ctl + C_GW2);
+  s.err = reinterpret_cast<int*>(s.ctl + C_ERR);
+  return s;
+}
+
+cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const double* anorm2,
+                           cudaStream_t st) {
+  const PreDims d = pre_dims(k, p);
+  cudaError_t err = cudaMemsetAsync(s.ctl, 0, C_WORDS * sizeof(int), st);
+  if (err != cudaSuccess) return err;
+  Pre32 a;
+  a.R = static_cast<float2*>(s.rows32);
+  a.V = a.R + (size_t)d.kp * d.pp;
+  a.k = k;
+  a.kp = d.kp;
+  a.pp = d.pp;
+  a.nb = d.kp / PB;
+  count_launches(1);
+  k_pre_init<<<grid_for((long long)d.kp * (d.pp + d.kp)), 256, 0, st>>>(R, p, anorm2, a);
+  // as many CTAs per pair as the SMs hold for all pairs at once (at least 8
+  // columns of R and 4 of V each)
+  const int pairs = a.nb / 2;
+  int C = 8, cap = 0;
+  for (;; C /= 2) {
+    a.pc = d.pp / C;
+    a.vc = d.kp / C;
+    a.chunk = a.pc + a.vc < kChunkMax ? a.pc + a.vc : kChunkMax;
+    err = cluster_capacity(C, a.chunk, &cap);
+    if (err != cudaSuccess) return err;
+    if (cap >= pairs || C == 1) break;
+  }
+  if (cap < 1) return cudaErrorInvalidConfiguration;
+  const int ncl = pairs < cap ? pairs : cap;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at[2];
+  launch_config(&cfg, at, ncl * C, C, kFixedSmem + (size_t)PM * (a.chunk + 2) * sizeof(float2), st,
+                true);
+  count_launches(1);
+  err = cudaLaunchKernelEx(&cfg, k_jacobi32, a, s.ctl);
+  if (err != cudaSuccess) return err;
+  count_launches(1);
+  k_pre_export<<<grid_for((long long)k * k), 256, 0, st>>>(a, s.K[0]);
+  return cudaGetLastError();
+}
+
+cudaError_t svd_pre_orth(const SvdPre& s, cplx* M, int k, int step, cudaStream_t st) {
+  count_launches(1);
+  k_pre_orth<<<k, RT, 0, st>>>(M, k, s.ctl, step);
+  return cudaGetLastError();
+}
+
+cudaError_t vec_copy_if(cplx* y, const cplx* x, long long n, const int* flag, bool want,
+                        cudaStream_t st) {
+  count_launches(1);
+  k_copy_if<<<grid_for(n), 256, 0, st>>>(y, x, n, reinterpret_cast<const unsigned int*>(flag),
+                                         want ? 1 : 0);
+  return cudaGetLastError();
+}
+
+cudaError_t svd_pre_corr(const SvdPre& s, const cplx* G, int k, double tol, const double* anorm2,
+                         double skip_rel, cplx* E, cudaStream_t st) {
+  count_launches(1);
+  k_pre_corr<<<k, RT, 0, st>>>(G, k, tol, anorm2, skip_rel, E, s.ctl);
+  return cudaGetLastError();
+}
+
+cudaError_t svd_pre_comb(const SvdPre& s, cplx* E, const cplx* W, const cplx* W2, int k,
+                         cudaStream_t st) {
+  const long long n = (long long)k * k;
+  count_launches(1);
+  k_pre_comb<<<grid_for(n), 256, 0, st>>>(E, W, W2, n, s.ctl);
+  return cudaGetLastError();
+}
+
+cudaError_t svd_pre_list(const SvdPre& s, const cplx* G, int k, double tol, const double* anorm2,
+                         double skip_rel, cudaStream_t st) {
+  int* flag = s.act + k + 1;
+  count_launches(2);
+  k_pre_flag<<<k, RT, 0, st>>>(G, k, tol, anorm2, skip_rel, flag, s.ctl);
+  k_pre_compact<<<1, 1024, 0, st>>>(flag, k, s.act);
+  return cudaGetLastError();
+}
+
+}  // namespace ite

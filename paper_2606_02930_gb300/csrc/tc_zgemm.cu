@@ -78,7 +78,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 k_zgemm_slices(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                int Mr, int N, int Kr, const int* __restrict__ eA, const int* __restrict__ eB,
                cplx* __restrict__ C, long long ldc, cplx alpha, cplx beta, const cplx* __restrict__ Z,
-               cplx gamma, int* err) {
+               cplx gamma, const int* run_if, int* err) {
+  if (run_if && *run_if == 0) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* stage_base = smem;
@@ -298,7 +299,9 @@ __device__ __forceinline__ __nv_bfloat16 bf(int v) { return __float2bfloat16_rn(
 // real rows 2r (Re, -Im interleaved) and 2r+1 (Im, Re), one warp per row r.
 // out: S blocks of (2M) x Kp bf16; eA[r] = row exponent.
 __global__ void k_slice_rows_A(const cplx* __restrict__ A, long long sAm, long long sAk, bool conj,
-                               int M, int K, int Kp, __nv_bfloat16* __restrict__ out, int* eA) {
+                               int M, int K, int Kp, __nv_bfloat16* __restrict__ out, int* eA,
+                               const int* run_if) {
+  if (run_if && *run_if == 0) return;
   const int r = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= M) return;
@@ -345,7 +348,9 @@ __global__ void k_slice_rows_A(const cplx* __restrict__ A, long long sAm, long l
 // K-major rows n: (Re, Im) interleaved along K.  One warp per column n.
 // out: S blocks of N x Kp bf16; eB[n] = column exponent.
 __global__ void k_slice_cols_B(const cplx* __restrict__ B, long long sBk, long long sBn, bool conj,
-                               int K, int N, int Kp, __nv_bfloat16* __restrict__ out, int* eB) {
+                               int K, int N, int Kp, __nv_bfloat16* __restrict__ out, int* eB,
+                               const int* run_if) {
+  if (run_if && *run_if == 0) return;
   const int n = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (n >= N) return;
@@ -429,11 +434,13 @@ cudaError_t zgemm_emu(const GemmArgs& g, void* scratch, size_t scratch_bytes, in
     const cplx* Zb = g.Z ? g.Z + (long long)b * g.sCb : nullptr;
     if (b == 0 || g.sAb != 0) {
       count_launches(1);
-      k_slice_rows_A<<<(g.M + 7) / 8, 256, 0, st>>>(A, g.sAm, g.sAk, g.conjA, g.M, g.K, (int)Kp, As, eA);
+      k_slice_rows_A<<<(g.M + 7) / 8, 256, 0, st>>>(A, g.sAm, g.sAk, g.conjA, g.M, g.K, (int)Kp, As, eA,
+                                                     g.run_if);
     }
     if (b == 0 || g.sBb != 0) {
       count_launches(1);
-      k_slice_cols_B<<<(g.N + 7) / 8, 256, 0, st>>>(B, g.sBk, g.sBn, g.conjB, g.K, g.N, (int)Kp, Bs, eB);
+      k_slice_cols_B<<<(g.N + 7) / 8, 256, 0, st>>>(B, g.sBk, g.sBn, g.conjB, g.K, g.N, (int)Kp, Bs, eB,
+                                                     g.run_if);
     }
     CUtensorMap ma, mb;
     cudaError_t e = make_digit_map(&ma, As, (long long)S * Mr, Kp, BM);
@@ -443,7 +450,7 @@ cudaError_t zgemm_emu(const GemmArgs& g, void* scratch, size_t scratch_bytes, in
     dim3 grid((g.N + BN - 1) / BN, (unsigned)((Mr + BM - 1) / BM));
     count_launches(1);
     k_zgemm_slices<<<grid, THREADS, smem, st>>>(ma, mb, (int)Mr, g.N, (int)Kp, eA, eB, Cb, g.ldc,
-                                                g.alpha, g.beta, Zb, g.gamma, err);
+                                                g.alpha, g.beta, Zb, g.gamma, g.run_if, err);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

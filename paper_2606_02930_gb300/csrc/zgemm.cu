@@ -18,6 +18,7 @@ __global__ void __launch_bounds__(THREADS)
 zgemm_kernel(GemmArgs g, bool a_kfast, bool b_nfast) {
   __shared__ cplx As[BK][BM + 1];
   __shared__ cplx Bs[BK][BN + 1];
+  if (g.run_if && *g.run_if == 0) return;
   const int t = threadIdx.x;
   const int tx = t % 16, ty = t / 16;
   const int row0 = blockIdx.y * BM, col0 = blockIdx.x * BN;
