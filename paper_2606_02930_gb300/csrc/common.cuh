@@ -110,8 +110,9 @@ cudaError_t heff_lp_apply(const void* ops, const MixPlan& plan2, int d, int D0, 
 
 // FP64-accurate complex GEMM on the bf16 tensor cores (exact 7-bit slicing,
 // see tc_zgemm.cu): same contract as zgemm; scratch of at least
-// zgemm_emu_scratch_bytes(M, N, K) bytes; *err set if a bounded wait ran out.
-size_t zgemm_emu_scratch_bytes(int M, int N, int K);
+// zgemm_emu_scratch_bytes(M, N, K, entries of A, of B) bytes (an operand shared by
+// the batch has one); *err set if a bounded wait ran out.
+size_t zgemm_emu_scratch_bytes(int M, int N, int K, int batchA = 1, int batchB = 1);
 cudaError_t zgemm_emu(const GemmArgs& g, void* scratch, size_t scratch_bytes, int* err,
                       cudaStream_t st);
 

@@ -294,7 +294,8 @@ ite_status gemm(ite_ctx ctx, int M, int N, int K, const cplx* A, long long sAm, 
   g.C = Cm; g.ldc = ldc; g.sCb = sCb;
   g.alpha = alpha; g.beta = beta; g.Z = Z; g.gamma = gamma;
   if (emulated(ctx, M, N, K)) {
-    CS(buf_ensure(ctx, ctx->ws_emu, zgemm_emu_scratch_bytes(M, N, K)));
+    CS(buf_ensure(ctx, ctx->ws_emu,
+                  zgemm_emu_scratch_bytes(M, N, K, sAb ? batch : 1, sBb ? batch : 1)));
     CK(zgemm_emu(g, ctx->ws_emu.p, ctx->ws_emu.n, reinterpret_cast<int*>(ctx->dcounter) + 10,
                  ctx->stream));
     return ITE_OK;

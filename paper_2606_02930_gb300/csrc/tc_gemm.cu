@@ -210,11 +210,24 @@ cudaError_t launch(const CUtensorMap& ma, const CUtensorMap& mb, float* C, int M
 
 }  // namespace
 
+// (k, row, batch entry, digit) of contiguous digit matrices: `digits` x `batch` x
+// `rows` x `cols` bf16, box (32, box_rows, 1, digits), 64-byte swizzle
 cudaError_t make_digit_map(CUtensorMap* map, const void* base, long long rows, long long cols,
-                           int box_rows) {
+                           int batch, int digits, int box_rows) {
   cudaError_t e = get_encoder();
   if (e != cudaSuccess) return e;
-  return make_map(map, base, rows, cols, cols, box_rows, 32);
+  if ((reinterpret_cast<uintptr_t>(base) & 15) || cols % 8 || cols < 1 || rows < 1)
+    return cudaErrorInvalidValue;
+  const cuuint64_t row = (cuuint64_t)(cols * 2);
+  cuuint64_t dims[4] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)batch, (cuuint64_t)digits};
+  cuuint64_t strides[3] = {row, row * rows, row * rows * batch};
+  cuuint32_t box[4] = {32, (cuuint32_t)box_rows, 1, (cuuint32_t)digits};
+  cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims,
+                        strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 cudaError_t tc_gemm_bf16(const void* A, long long lda, const void* B, long long ldb, float* C,
