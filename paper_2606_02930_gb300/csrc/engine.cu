@@ -47,7 +47,7 @@ constexpr int kMaxKrylov = 32;
 constexpr double kEmuMinWork = 2.0e6;    // complex MACs below which GEMMs stay native
 // Rows from which the Jacobi of a split is preconditioned.  A whole split of k x k,
 // without and with it: k = 16 0.81 and 0.70 ms, 24 1.36 and 0.91, 32 2.00 and
-// 1.05, 64 4.36 and 2.05, 128 9.14 and 3.48, 512 69.7 and 22.6.  Below 16 rows
+// 1.05, 64 4.36 and 1.80, 512 69.9 and 13.9.  Below 16 rows
 // one cluster step covers the whole matrix and the GEMMs' launches outweigh the
 // few rounds saved.
 constexpr int kPreMinRows = 16;

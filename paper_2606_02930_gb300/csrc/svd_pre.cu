@@ -40,7 +40,7 @@ namespace ite {
 namespace {
 
 // control words (PreCtl in device memory, cleared before each use)
-constexpr int C_ARRIVE = 0, C_GEN = 1, C_ERR = 4, C_SWEEPS = 5;
+constexpr int C_ARRIVE = 0, C_ERR = 4, C_SWEEPS = 5;
 constexpr int C_OK = 8, C_GE = 9, C_GW = 10, C_GW2 = 11, C_COUNT = 12, C_GN = 13;
 constexpr int C_DELTA = 16, C_NU = 18;        // 64-bit words
 constexpr int C_OFF = 24;                     // per-sweep largest overlap (float bits)
@@ -58,46 +58,85 @@ constexpr float kRot32 = 2e-7f;               // overlaps below this are fp32 ro
 constexpr float kTiny32 = 1e-34f;             // squared norms below this (of 1) are left alone
 
 struct Pre32 {
-  float2* R;                                  // kp x pp, the scaled rows
-  float2* V;                                  // kp x kp, the accumulated rotation
-  int k, kp, pp, nb;                          // rows, padded rows, padded length, blocks
+  float2* R;                                  // kp rows of pl, the scaled rows of R
+  float2* V;                                  // kp rows of vl, the accumulated rotation
+  int k, kp, pl, vl, nb;                      // rows, padded rows, row strides, blocks
   int pc, vc, chunk;                          // columns of R and V per CTA, columns staged at once
 };
 
-// Barrier over the clusters' first CTAs; bounded like grid_barrier (svd.cu).
-__device__ bool leader_barrier(unsigned int* st, unsigned int n) {
-  volatile unsigned int* gen = st + C_GEN;
-  const unsigned int g = *gen;
-  __threadfence();
-  if (atomicAdd(st + C_ARRIVE, 1u) == n - 1) {
-    atomicExch(st + C_ARRIVE, 0u);
-    __threadfence();
-    atomicAdd(st + C_GEN, 1u);
-  } else {
-    unsigned long long spins = 0;
-    while (*gen == g) {
-      if (*((volatile unsigned int*)(st + C_ERR)) != 0u) break;
-      if (++spins > (1ull << 24)) {
-        atomicExch(st + C_ERR, 1u);
-        break;
-      }
-      __nanosleep(20);
+// Barrier over the clusters' first CTAs: arrivals are counted up without a reset,
+// barrier number t is passed at t n of them (one trip to L2 to arrive, one to
+// see it).  Bounded: after 2^24 polls the error flag is set, and a wait also
+// gives up as soon as another has set it.
+__device__ bool leader_barrier(unsigned int* st, unsigned int target) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(st + C_ARRIVE) : "memory");
+  unsigned long long spins = 0;
+  for (;;) {
+    unsigned int seen;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(st + C_ARRIVE) : "memory");
+    if ((int)(seen - target) >= 0) return true;
+    if (*((volatile unsigned int*)(st + C_ERR)) != 0u) return false;
+    if (++spins > (1ull << 24)) {
+      atomicExch(st + C_ERR, 1u);
+      return false;
     }
   }
-  __threadfence();
-  return *((volatile unsigned int*)(st + C_ERR)) == 0u;
 }
 
 __device__ __forceinline__ int seat(int pos, int round, int n) {
   return pos == 0 ? 0 : ((pos - 1 + round) % (n - 1)) + 1;
 }
 
-// Local column c of this CTA in the concatenated row [R | V] (two columns at
-// a time: pc and vc are even).
+// Local column c of this CTA in the concatenated row [R | V] (aligned pairs of
+// columns: pc and vc are multiples of 4).
 __device__ __forceinline__ float4* col_ptr(const Pre32& a, int row, int rank, int c) {
-  float2* p = c < a.pc ? a.R + (long long)row * a.pp + (long long)rank * a.pc + c
-                       : a.V + (long long)row * a.kp + (long long)rank * a.vc + (c - a.pc);
+  float2* p = c < a.pc ? a.R + (long long)row * a.pl + (long long)rank * a.pc + c
+                       : a.V + (long long)row * a.vl + (long long)rank * a.vc + (c - a.pc);
   return reinterpret_cast<float4*>(p);
+}
+
+__device__ __forceinline__ void copy16(float2* dst, const float4* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                   (unsigned int)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// Rotation x' = c x - s y, y' = conj(s) x + c y of two rows with squared norms
+// al, be and inner product g = x y^H that makes them orthogonal; returns what it
+// moves from al to be.  Written in the overlap h = g / (|x| |y|) and the ratio of
+// the norms, which stay in range for rows of any weight, and in approximate
+// reciprocals and square roots (the chain of them is what a round waits for);
+// c is refined by a Newton step so that |c|^2 + |s|^2 = 1 to rounding.
+__device__ __forceinline__ float rotation(float al, float be, float2 g, float& c, float& sx,
+                                          float& sy, float& off) {
+  c = 1.f;
+  sx = sy = 0.f;
+  if (!(al > kTiny32 && be > kTiny32)) return 0.f;
+  const float ra = rsqrtf(al), rb = rsqrtf(be);
+  const float hx = g.x * ra * rb, hy = g.y * ra * rb;
+  const float h2 = fmaf(hx, hx, hy * hy);
+  if (!(h2 > kRot32 * kRot32)) return 0.f;
+  const float ih = rsqrtf(h2), h = h2 * ih;
+  off = fmaxf(off, h);
+  // zeta = (be - al) / (2 |g|), tangent t = 1 / (|zeta| + sqrt(1 + zeta^2))
+  const float q = be * rb * ra, qi = al * ra * rb;
+  const float z = 0.5f * (q - qi) * ih, az = fabsf(z);
+  const float w = fmaf(z, z, 1.f);
+  const float t = rcp_approx(az < 1e9f ? az + w * rsqrtf(w) : az + az);
+  const float d = fmaf(t, t, 1.f);
+  c = rsqrtf(d);
+  c = c * fmaf(-0.5f * d * c, c, 1.5f);
+  const float sg = copysignf(c * t * ih, z);
+  sx = sg * hx;
+  sy = sg * hy;
+  return copysignf(t * h * (al * ra) * (be * rb), z);
 }
 
 // One cluster per block pair, the columns of the pair's rows dealt to its
@@ -105,13 +144,14 @@ __device__ __forceinline__ float4* col_ptr(const Pre32& a, int row, int rank, in
 // Gram matrix, the shares are added through distributed shared memory in a
 // fixed order, every CTA diagonalises the sum the same way and applies the
 // result to its own columns.
-// Bound: latency.  A step of the k = 512 case moves 8 MB through L2 and does
-// 50 MFLOP on 128 SMs (2 us); the 31 dependent rounds of the 32 x 32
-// diagonalisation take most of the rest.  16-row blocks: 8-row ones need
-// twice the steps and barriers for the same number of rounds, 32-row ones
-// leave half the SMs without a pair.  Whole 512 x 512 split (chi_max 256, cutoff
-// 1e-10): 69.3 ms with the FP64 Jacobi alone, 22.6 ms with the preconditioner
-// (none of the FP64 sweeps is left); 1024 x 1024: 324 ms and 79 ms.
+// Bound: latency and shared memory.  Clocks per step at k = 512 (16 pairs, 6 CTAs
+// each, 31 steps a sweep): copy in 2.2k, Gram 5.8k, sum 3.8k, the 16 or 31
+// dependent rounds 18k (900 each: the chain of approximate square roots, then
+// the two-sided update), rows 12k, grid barrier 6.9k; 23.7 us in all.  16-row
+// blocks: 8-row ones need twice the steps and barriers for the same number of
+// rounds, 32-row ones leave half the SMs without a pair.  Whole 512 x 512 split
+// (chi_max 256, cutoff 1e-10): 69.9 ms with the FP64 Jacobi alone, 13.9 ms with
+// the preconditioner (no FP64 sweep is left); 1024 x 1024: 325 ms and 54.6 ms.
 __global__ void __launch_bounds__(PT)
 k_jacobi32(Pre32 a, unsigned int* st) {
   cg::cluster_group cl = cg::this_cluster();
@@ -121,23 +161,30 @@ k_jacobi32(Pre32 a, unsigned int* st) {
   extern __shared__ float4 dyn[];
   float2* part = reinterpret_cast<float2*>(dyn);            // PM x GLD
   float2* G = part + PM * GLD;                              // PM x GLD
-  float2* QT = G + PM * GLD;                                // PM x QLD: QT[c][r] = Q[r][c]
+  float2* G2 = G + PM * GLD;                                // PM x GLD
+  float2* QT = G2 + PM * GLD;                               // PM x QLD: QT[c][r] = Q[r][c]
   float2* S = QT + PM * QLD;                                // PM x ld
-  __shared__ float4 rot[PB];
   __shared__ int s_pos[PM];
   __shared__ int s_off, s_ok;
   const int lc = a.pc + a.vc, ld = a.chunk + 2;
   const bool resident = lc <= a.chunk;
   const int ty = tid >> 4, tx = tid & 15;
+  unsigned int passed = 0;                    // barrier arrivals so far
+  // the two row pairs pa < pb whose block of G this thread turns (tid < 120):
+  // rows x and 15 - x of the 16 x 16 triangle make one row of 15 blocks
+  const int fx = min(tid, 119) / 15, fy = min(tid, 119) - 15 * fx;
+  const int pa = fy >= fx ? fx : 15 - fx, pb = fy >= fx ? fy + 1 : 16 - fx + fy;
 
-  // rows of the pair (u, v): 0..15 of block u, then 0..15 of block v
+  // rows of the pair (u, v): 0..15 of block u, then 0..15 of block v; each warp
+  // copies four rows
   auto stage = [&](int u, int v, int c0, int n) {
-    const int n2 = n >> 1;
-    for (int e = tid; e < PM * n2; e += PT) {
-      const int r = e / n2, c = 2 * (e - r * n2);
-      const int row = (r < PB ? u * PB + r : v * PB + r - PB);
-      *reinterpret_cast<float4*>(S + r * ld + c) = __ldcg(col_ptr(a, row, rank, c0 + c));
-    }
+    const int r0 = 4 * warp;
+    const int row = (r0 < PB ? u * PB : (v - 1) * PB) + r0;
+    for (int c = 2 * lane; c < n; c += 64)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        copy16(S + (r0 + i) * ld + c, col_ptr(a, row + i, rank, c0 + c));
+    asm volatile("cp.async.wait_all;" ::: "memory");
   };
 
   for (int sw = 0; sw < kSweeps32; ++sw) {
@@ -167,8 +214,8 @@ k_jacobi32(Pre32 a, unsigned int* st) {
 #pragma unroll
             for (int i = 0; i < 2; ++i)
 #pragma unroll
-              for (int j = 0; j < 2; ++j) {
-                // x conj(y)
+              for (int j = i; j < 2; ++j) {
+                // x conj(y) (rows ty + 16 by tx mirror others' ty by tx + 16)
                 acc[i][j].x = fmaf(x[i].x, y[j].x, fmaf(x[i].y, y[j].y, acc[i][j].x));
                 acc[i][j].y = fmaf(x[i].y, y[j].x, fmaf(-x[i].x, y[j].y, acc[i][j].y));
                 acc[i][j].x = fmaf(x[i].z, y[j].z, fmaf(x[i].w, y[j].w, acc[i][j].x));
@@ -180,133 +227,127 @@ k_jacobi32(Pre32 a, unsigned int* st) {
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
-          for (int j = 0; j < 2; ++j) part[(ty + PB * i) * GLD + tx + PB * j] = acc[i][j];
+          for (int j = i; j < 2; ++j) part[(ty + PB * i) * GLD + tx + PB * j] = acc[i][j];
         cl.sync();
         // ---- sum of the shares (upper triangle, mirrored); Q = I
-        for (int e = tid; e < PM * PM; e += PT) {
-          const int i = e / PM, j = e - i * PM;
-          if (i <= j) {
-            float2 s = make_float2(0.f, 0.f);
-            for (int r = 0; r < C; ++r) {
-              const float2 t = cl.map_shared_rank(part, r)[i * GLD + j];
-              s.x += t.x;
-              s.y += t.y;
-            }
-            if (i == j) {
-              // padding rows sort last and never rotate
-              const int row = i < PB ? u * PB + i : v * PB + i - PB;
-              G[i * GLD + i] = make_float2(row < a.k ? s.x : -1.f, 0.f);
-            } else {
-              G[i * GLD + j] = s;
-              G[j * GLD + i] = make_float2(s.x, -s.y);
-            }
+        for (int e = tid; e < PM * (PM + 1) / 2; e += PT) {
+          // rows x and 31 - x of the triangle make one row of 33 entries
+          const int x = e / (PM + 1), y = e - x * (PM + 1);
+          const int i = y > x ? x : PM - 1 - x, j = y > x ? y - 1 : PM - 1 - y;
+          float2 t[8];
+#pragma unroll
+          for (int r = 0; r < 8; ++r)
+            t[r] = r < C ? cl.map_shared_rank(part, r)[i * GLD + j] : make_float2(0.f, 0.f);
+          float2 s = t[0];
+#pragma unroll
+          for (int r = 1; r < 8; ++r) {
+            s.x += t[r].x;
+            s.y += t[r].y;
           }
-          QT[i * QLD + j] = make_float2(i == j ? 1.f : 0.f, 0.f);
+          if (i == j) {
+            // padding rows sort last and never rotate
+            const int row = i < PB ? u * PB + i : v * PB + i - PB;
+            G[i * GLD + i] = make_float2(row < a.k ? s.x : -1.f, 0.f);
+          } else {
+            G[i * GLD + j] = s;
+            G[j * GLD + i] = make_float2(s.x, -s.y);
+          }
         }
+        for (int e = tid; e < PM * PM; e += PT)
+          QT[(e >> 5) * QLD + (e & 31)] = make_float2((e >> 5) == (e & 31) ? 1.f : 0.f, 0.f);
         if (tid == 0) s_off = 0;
         __syncthreads();
-        // ---- one cyclic sweep of rotations: thread t < 16 forms those of the round
+        // ---- one cyclic sweep of rotations, all pairs of the 32 rows in every
+        // fourth step, only those across the two blocks (16 rounds instead of
+        // 31) in the others: as many sweeps as with all pairs every time.
+        // Round r pairs row i with row i ^ r; pair t is the t-th i whose highest
+        // bit of r is clear.  Lane t of every warp forms the rotation of pair
+        // t.  Warps 0-3 turn the 120 blocks of two different pairs from one copy
+        // of G to the other (upper block, mirrored), warps 4-7 the rows of Q
+        // and the pairs' own blocks, so one barrier a round is enough.
         float off = 0.f;
-        for (int r = 0; r < PM - 1; ++r) {
-          if (tid < PB) {
-            int i = seat(tid, r, PM), j = seat(PM - 1 - tid, r, PM);
-            if (i > j) { const int t = i; i = j; j = t; }
-            const float al = G[i * GLD + i].x, be = G[j * GLD + j].x;
-            const float2 g = G[i * GLD + j];
-            float c = 1.f, sx = 0.f, sy = 0.f, tg = 0.f;
-            if (al > kTiny32 && be > kTiny32) {
-              // the overlap (hx, hy) = g / (|x| |y|): its square stays in range
-              // for rows of any weight
-              const float ra = rsqrtf(al), rb = rsqrtf(be);
-              const float hx = g.x * ra * rb, hy = g.y * ra * rb;
-              const float h2 = fmaf(hx, hx, hy * hy);
-              if (h2 > kRot32 * kRot32) {
-                const float ih = rsqrtf(h2), h = h2 * ih;
-                off = fmaxf(off, h);
-                // tangent of the rotation that zeroes g, |t| <= 1
-                const float ga = h * (al * ra) * (be * rb);
-                const float D = be - al, z = fabsf(D) / (2.f * ga);
-                const float t = 1.f / (z + sqrtf(fmaf(z, z, 1.f)));
-                const float q = fmaf(t, t, 1.f);
-                c = rsqrtf(q);
-                c = c * fmaf(-0.5f * q * c, c, 1.5f);
-                const float sg = (D >= 0.f ? c * t : -c * t) * ih;
-                sx = sg * hx;
-                sy = sg * hy;
-                tg = D >= 0.f ? t * ga : -t * ga;
-              }
-            }
-            rot[tid] = make_float4(c, sx, sy, tg);
-          }
-          __syncthreads();
-          {
-            // thread (ty, tx): the 2 x 2 block of row pair ty and column pair tx
-            int i = seat(ty, r, PM), j = seat(PM - 1 - ty, r, PM);
-            if (i > j) { const int t = i; i = j; j = t; }
-            int m = seat(tx, r, PM), n = seat(PM - 1 - tx, r, PM);
-            if (m > n) { const int t = m; m = n; n = t; }
-            const float4 ra = rot[ty], rb = rot[tx];
-            if (ty == tx) {
-              if (ra.y != 0.f || ra.z != 0.f) {
-                G[i * GLD + i].x -= ra.w;
-                G[j * GLD + j].x += ra.w;
-                G[i * GLD + j] = G[j * GLD + i] = make_float2(0.f, 0.f);
-              }
-            } else {
-              const float2 b00 = G[i * GLD + m], b01 = G[i * GLD + n];
-              const float2 b10 = G[j * GLD + m], b11 = G[j * GLD + n];
+        float2 *Ga = G, *Gb = G2;
+        for (int r = (rd & 3) == 0 ? 1 : PB; r < PM; ++r) {
+          const int hb = 31 - __clz(r), low = (1 << hb) - 1;
+          auto first = [&](int t) { return ((t & ~low) << 1) | (t & low); };
+          const int m = first(tx), n = m ^ r;
+          const float al = Ga[m * GLD + m].x, be = Ga[n * GLD + n].x;
+          const float2 g = Ga[m * GLD + n];
+          if (warp < 4) {
+            const int i = first(pa), j = i ^ r, k2 = first(pb), l2 = k2 ^ r;
+            const float2 b00 = Ga[i * GLD + k2], b01 = Ga[i * GLD + l2];
+            const float2 b10 = Ga[j * GLD + k2], b11 = Ga[j * GLD + l2];
+            float c, sx, sy;
+            rotation(al, be, g, c, sx, sy, off);
+            const float ca = __shfl_sync(0xffffffffu, c, pa), cb = __shfl_sync(0xffffffffu, c, pb);
+            const float xa = __shfl_sync(0xffffffffu, sx, pa), xb = __shfl_sync(0xffffffffu, sx, pb);
+            const float ya = __shfl_sync(0xffffffffu, sy, pa), yb = __shfl_sync(0xffffffffu, sy, pb);
+            if (tid < 120) {
               // rows: x' = c x - s y, y' = conj(s) x + c y
               float2 p00, p01, p10, p11;
-              p00.x = ra.x * b00.x - (ra.y * b10.x - ra.z * b10.y);
-              p00.y = ra.x * b00.y - (ra.y * b10.y + ra.z * b10.x);
-              p01.x = ra.x * b01.x - (ra.y * b11.x - ra.z * b11.y);
-              p01.y = ra.x * b01.y - (ra.y * b11.y + ra.z * b11.x);
-              p10.x = (ra.y * b00.x + ra.z * b00.y) + ra.x * b10.x;
-              p10.y = (ra.y * b00.y - ra.z * b00.x) + ra.x * b10.y;
-              p11.x = (ra.y * b01.x + ra.z * b01.y) + ra.x * b11.x;
-              p11.y = (ra.y * b01.y - ra.z * b01.x) + ra.x * b11.y;
+              p00.x = ca * b00.x - (xa * b10.x - ya * b10.y);
+              p00.y = ca * b00.y - (xa * b10.y + ya * b10.x);
+              p01.x = ca * b01.x - (xa * b11.x - ya * b11.y);
+              p01.y = ca * b01.y - (xa * b11.y + ya * b11.x);
+              p10.x = (xa * b00.x + ya * b00.y) + ca * b10.x;
+              p10.y = (xa * b00.y - ya * b00.x) + ca * b10.y;
+              p11.x = (xa * b01.x + ya * b01.y) + ca * b11.x;
+              p11.y = (xa * b01.y - ya * b01.x) + ca * b11.y;
               // columns: x' = c x - conj(s) y, y' = s x + c y
-              float2 o;
-              o.x = rb.x * p00.x - (rb.y * p01.x + rb.z * p01.y);
-              o.y = rb.x * p00.y - (rb.y * p01.y - rb.z * p01.x);
-              G[i * GLD + m] = o;
-              o.x = (rb.y * p00.x - rb.z * p00.y) + rb.x * p01.x;
-              o.y = (rb.y * p00.y + rb.z * p00.x) + rb.x * p01.y;
-              G[i * GLD + n] = o;
-              o.x = rb.x * p10.x - (rb.y * p11.x + rb.z * p11.y);
-              o.y = rb.x * p10.y - (rb.y * p11.y - rb.z * p11.x);
-              G[j * GLD + m] = o;
-              o.x = (rb.y * p10.x - rb.z * p10.y) + rb.x * p11.x;
-              o.y = (rb.y * p10.y + rb.z * p10.x) + rb.x * p11.y;
-              G[j * GLD + n] = o;
+              auto put = [&](int row, int col, float x, float y) {
+                Gb[row * GLD + col] = make_float2(x, y);
+                Gb[col * GLD + row] = make_float2(x, -y);
+              };
+              put(i, k2, cb * p00.x - (xb * p01.x + yb * p01.y), cb * p00.y - (xb * p01.y - yb * p01.x));
+              put(i, l2, (xb * p00.x - yb * p00.y) + cb * p01.x, (xb * p00.y + yb * p00.x) + cb * p01.y);
+              put(j, k2, cb * p10.x - (xb * p11.x + yb * p11.y), cb * p10.y - (xb * p11.y - yb * p11.x));
+              put(j, l2, (xb * p10.x - yb * p10.y) + cb * p11.x, (xb * p10.y + yb * p10.x) + cb * p11.y);
             }
-            // rows m, n of Q, columns ty and ty + 16
+          } else {
+            // rows m, n of Q, four columns of it
+            float2* const q = QT + (2 * (warp - 4) + (lane >> 4)) * QLD;
+            float2 x[4], y[4];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              float2* q = QT + (ty + PB * h) * QLD;
-              const float2 x = q[m], y = q[n];
-              q[m] = make_float2(rb.x * x.x - (rb.y * y.x - rb.z * y.y),
-                                 rb.x * x.y - (rb.y * y.y + rb.z * y.x));
-              q[n] = make_float2((rb.y * x.x + rb.z * x.y) + rb.x * y.x,
-                                 (rb.y * x.y - rb.z * x.x) + rb.x * y.y);
+            for (int h = 0; h < 4; ++h) {
+              x[h] = q[8 * h * QLD + m];
+              y[h] = q[8 * h * QLD + n];
+            }
+            float c, sx, sy;
+            const float d = rotation(al, be, g, c, sx, sy, off);
+            if (warp == 4 && lane < PB) {
+              const float2 z = sx != 0.f || sy != 0.f ? make_float2(0.f, 0.f) : g;
+              Gb[m * GLD + m] = make_float2(al - d, 0.f);
+              Gb[n * GLD + n] = make_float2(be + d, 0.f);
+              Gb[m * GLD + n] = z;
+              Gb[n * GLD + m] = make_float2(z.x, -z.y);
+            }
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+              q[8 * h * QLD + m] = make_float2(c * x[h].x - (sx * y[h].x - sy * y[h].y),
+                                               c * x[h].y - (sx * y[h].y + sy * y[h].x));
+              q[8 * h * QLD + n] = make_float2((sx * x[h].x + sy * x[h].y) + c * y[h].x,
+                                               (sx * x[h].y - sy * x[h].x) + c * y[h].y);
             }
           }
           __syncthreads();
+          float2* const t = Ga;
+          Ga = Gb;
+          Gb = t;
         }
         if (tid < PB) atomicMax(&s_off, __float_as_int(off));
         // ---- heavier rows first
         if (tid < PM) {
-          const float di = G[tid * GLD + tid].x;
+          const float di = Ga[tid * GLD + tid].x;
           int pos = 0;
           for (int j = 0; j < PM; ++j) {
-            const float dj = G[j * GLD + j].x;
+            const float dj = Ga[j * GLD + j].x;
             pos += (dj > di) || (dj == di && j < tid);
           }
           s_pos[tid] = pos;
         }
         __syncthreads();
         if (tid == 0 && rank == 0) atomicMax(st + C_OFF + sw, (unsigned int)s_off);
-        // ---- rows <- Q rows: warp w the rows 8 (w % 4).., 64 columns at a time
+        // ---- rows <- Q rows: warp w the rows 8 (w % 4).., 32 columns at a time
         const int r0 = 8 * (warp & 3);
         for (int c0 = 0; c0 < lc; c0 += a.chunk) {
           const int n = min(a.chunk, lc - c0);
@@ -315,30 +356,26 @@ k_jacobi32(Pre32 a, unsigned int* st) {
             stage(u, v, c0, n);
             __syncthreads();
           }
-          for (int cb = (warp >> 2) * 64; cb < n; cb += 128) {
-            const int c = cb + 2 * lane;
+          for (int cb = (warp >> 2) * 32; cb < n; cb += 64) {
+            const int c = cb + lane;
             const bool in = c < n;
             const float2* sp = S + (in ? c : 0);
-            float2 o[8][2];
+            float2 o[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) o[i][0] = o[i][1] = make_float2(0.f, 0.f);
-#pragma unroll 4
+            for (int i = 0; i < 8; ++i) o[i] = make_float2(0.f, 0.f);
+#pragma unroll 8
             for (int m = 0; m < PM; ++m) {
-              const float4 s = *reinterpret_cast<const float4*>(sp + m * ld);
+              const float2 s = sp[m * ld];
               const float4* qp = reinterpret_cast<const float4*>(QT + m * QLD + r0);
 #pragma unroll
               for (int i2 = 0; i2 < 4; ++i2) {
                 const float4 q = qp[i2];
-                float2* o0 = o[2 * i2];
-                float2* o1 = o[2 * i2 + 1];
-                o0[0].x = fmaf(q.x, s.x, fmaf(-q.y, s.y, o0[0].x));
-                o0[0].y = fmaf(q.x, s.y, fmaf(q.y, s.x, o0[0].y));
-                o0[1].x = fmaf(q.x, s.z, fmaf(-q.y, s.w, o0[1].x));
-                o0[1].y = fmaf(q.x, s.w, fmaf(q.y, s.z, o0[1].y));
-                o1[0].x = fmaf(q.z, s.x, fmaf(-q.w, s.y, o1[0].x));
-                o1[0].y = fmaf(q.z, s.y, fmaf(q.w, s.x, o1[0].y));
-                o1[1].x = fmaf(q.z, s.z, fmaf(-q.w, s.w, o1[1].x));
-                o1[1].y = fmaf(q.z, s.w, fmaf(q.w, s.z, o1[1].y));
+                float2& o0 = o[2 * i2];
+                float2& o1 = o[2 * i2 + 1];
+                o0.x = fmaf(q.x, s.x, fmaf(-q.y, s.y, o0.x));
+                o0.y = fmaf(q.x, s.y, fmaf(q.y, s.x, o0.y));
+                o1.x = fmaf(q.z, s.x, fmaf(-q.w, s.y, o1.x));
+                o1.y = fmaf(q.z, s.y, fmaf(q.w, s.x, o1.y));
               }
             }
             if (in) {
@@ -346,8 +383,7 @@ k_jacobi32(Pre32 a, unsigned int* st) {
               for (int i = 0; i < 8; ++i) {
                 const int pos = s_pos[r0 + i];
                 const int row = pos < PB ? u * PB + pos : v * PB + pos - PB;
-                *col_ptr(a, row, rank, c0 + c) =
-                    make_float4(o[i][0].x, o[i][0].y, o[i][1].x, o[i][1].y);
+                *reinterpret_cast<float2*>(col_ptr(a, row, rank, c0 + c)) = o[i];
               }
             }
           }
@@ -356,7 +392,8 @@ k_jacobi32(Pre32 a, unsigned int* st) {
         cl.sync();
       }
       cl.sync();
-      if (rank == 0 && tid == 0) s_ok = leader_barrier(st, (unsigned int)ncl) ? 1 : 0;
+      passed += (unsigned int)ncl;
+      if (rank == 0 && tid == 0) s_ok = leader_barrier(st, passed) ? 1 : 0;
       cl.sync();
       ok = *cl.map_shared_rank(&s_ok, 0) != 0;
       if (!ok) break;
@@ -372,19 +409,19 @@ k_jacobi32(Pre32 a, unsigned int* st) {
 __global__ void k_pre_init(const cplx* __restrict__ R, int p, const double* anorm2, Pre32 a) {
   const double n2 = *anorm2;
   const double s = n2 > 0.0 && isfinite(n2) ? rsqrt(n2) : 0.0;
-  const long long w = a.pp + a.kp, tot = w * a.kp;
+  const long long w = a.pl + a.vl, tot = w * a.kp;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
        e += (long long)gridDim.x * blockDim.x) {
     const int i = (int)(e / w), c = (int)(e - (long long)i * w);
-    if (c < a.pp) {
+    if (c < a.pl) {
       float2 v = make_float2(0.f, 0.f);
       if (i < a.k && c < p) {
         const cplx x = R[(long long)i * p + c];
         v = make_float2((float)(x.x * s), (float)(x.y * s));
       }
-      a.R[(long long)i * a.pp + c] = v;
+      a.R[(long long)i * a.pl + c] = v;
     } else {
-      a.V[(long long)i * a.kp + c - a.pp] = make_float2(i == c - a.pp ? 1.f : 0.f, 0.f);
+      a.V[(long long)i * a.vl + c - a.pl] = make_float2(i == c - a.pl ? 1.f : 0.f, 0.f);
     }
   }
 }
@@ -394,7 +431,7 @@ __global__ void k_pre_export(Pre32 a, cplx* __restrict__ V) {
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
        e += (long long)gridDim.x * blockDim.x) {
     const int i = (int)(e / a.k), c = (int)(e - (long long)i * a.k);
-    const float2 v = a.V[(long long)i * a.kp + c];
+    const float2 v = a.V[(long long)i * a.vl + c];
     V[e] = cmake(v.x, v.y);
   }
 }
@@ -583,20 +620,27 @@ int grid_for(long long tot) {
 
 long long round_up(long long x, long long m) { return (x + m - 1) / m * m; }
 
+// Padded rows, and row strides that leave room for the last CTA's share of
+// columns (a multiple of 4 per CTA, up to 8 CTAs).
 struct PreDims {
-  int kp, pp;
+  int kp, pl, vl;
 };
-PreDims pre_dims(int k, int p) { return {(int)round_up(k, PM), (int)round_up(p, 32)}; }
+PreDims pre_dims(int k, int p) {
+  const int kp = (int)round_up(k, PM);
+  return {kp, (int)round_up(p, 4) + 32, kp + 32};
+}
+int share(int columns, int C) { return 4 * ((columns + 4 * C - 1) / (4 * C)); }
 
-constexpr size_t kFixedSmem = (size_t)PM * (2 * GLD + QLD) * sizeof(float2);
+constexpr size_t kFixedSmem = (size_t)PM * (3 * GLD + QLD) * sizeof(float2);
 constexpr int kChunkMax = 640;                // columns staged at once: 32 x 642 x 8 B = 164 KB
+constexpr size_t kOwnSmSmem = 116 * 1024;     // more than half of an SM's shared memory
 
 // Clusters of C CTAs with this much shared memory that can be resident at
-// once on the current device, cached per (device, C, columns); several host
+// once on the current device, cached per (device, C, bytes); several host
 // threads may ask at once.
 struct ClusterCapacity {
   std::mutex mu;
-  struct Entry { int dev, C, chunk, n; };
+  struct Entry { int dev, C; size_t smem; int n; };
   Entry e[64];
   int used = 0;
 } g_cap;
@@ -617,17 +661,16 @@ void launch_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int grid, i
   cfg->numAttrs = coop ? 2 : 1;
 }
 
-cudaError_t cluster_capacity(int C, int chunk, int* n) {
+cudaError_t cluster_capacity(int C, size_t smem, int* n) {
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
   std::lock_guard<std::mutex> lock(g_cap.mu);
   for (int i = 0; i < g_cap.used; ++i)
-    if (g_cap.e[i].dev == dev && g_cap.e[i].C == C && g_cap.e[i].chunk == chunk) {
+    if (g_cap.e[i].dev == dev && g_cap.e[i].C == C && g_cap.e[i].smem == smem) {
       *n = g_cap.e[i].n;
       return cudaSuccess;
     }
-  const size_t smem = kFixedSmem + (size_t)PM * (chunk + 2) * sizeof(float2);
   err = cudaFuncSetAttribute(k_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(kFixedSmem + (size_t)PM * (kChunkMax + 2) * sizeof(float2)));
   if (err != cudaSuccess) return err;
@@ -636,7 +679,7 @@ cudaError_t cluster_capacity(int C, int chunk, int* n) {
   launch_config(&cfg, at, C * 1024, C, smem, nullptr, false);
   err = cudaOccupancyMaxActiveClusters(n, k_jacobi32, &cfg);
   if (err != cudaSuccess) return err;
-  if (g_cap.used < 64) g_cap.e[g_cap.used++] = {dev, C, chunk, *n};
+  if (g_cap.used < 64) g_cap.e[g_cap.used++] = {dev, C, smem, *n};
   return cudaSuccess;
 }
 
@@ -644,7 +687,7 @@ cudaError_t cluster_capacity(int C, int chunk, int* n) {
 
 size_t svd_pre_bytes(int k, int p) {
   const PreDims d = pre_dims(k, p);
-  return (size_t)d.kp * (d.pp + d.kp) * sizeof(float2) + 4 * (size_t)k * k * sizeof(cplx) +
+  return (size_t)d.kp * (d.pl + d.vl) * sizeof(float2) + 4 * (size_t)k * k * sizeof(cplx) +
          (size_t)(2 * k + 1) * sizeof(int) + C_WORDS * sizeof(int) + 6 * 256;
 }
 
@@ -657,7 +700,7 @@ SvdPre svd_pre_carve(void* ws, int k, int p) {
     c += round_up((long long)bytes, 256);
     return r;
   };
-  s.rows32 = take((size_t)d.kp * (d.pp + d.kp) * sizeof(float2));
+  s.rows32 = take((size_t)d.kp * (d.pl + d.vl) * sizeof(float2));
   for (cplx*& m : s.K) m = reinterpret_cast<cplx*>(take((size_t)k * k * sizeof(cplx)));
   s.act = reinterpret_cast<int*>(take((size_t)(2 * k + 1) * sizeof(int)));
   s.ctl = reinterpret_cast<unsigned int*>(take(C_WORDS * sizeof(int)));
@@ -677,22 +720,26 @@ cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const d
   if (err != cudaSuccess) return err;
   Pre32 a;
   a.R = static_cast<float2*>(s.rows32);
-  a.V = a.R + (size_t)d.kp * d.pp;
+  a.V = a.R + (size_t)d.kp * d.pl;
   a.k = k;
   a.kp = d.kp;
-  a.pp = d.pp;
+  a.pl = d.pl;
+  a.vl = d.vl;
   a.nb = d.kp / PB;
   count_launches(1);
-  k_pre_init<<<grid_for((long long)d.kp * (d.pp + d.kp)), 256, 0, st>>>(R, p, anorm2, a);
-  // as many CTAs per pair as the SMs hold for all pairs at once (at least 8
-  // columns of R and 4 of V each)
+  k_pre_init<<<grid_for((long long)d.kp * (d.pl + d.vl)), 256, 0, st>>>(R, p, anorm2, a);
+  // as many CTAs per pair as give every CTA an SM of its own (two on one SM
+  // take turns at every phase of the step)
   const int pairs = a.nb / 2;
   int C = 8, cap = 0;
-  for (;; C /= 2) {
-    a.pc = d.pp / C;
-    a.vc = d.kp / C;
+  size_t smem = 0;
+  for (;; --C) {
+    a.pc = share(p, C);
+    a.vc = share(d.kp, C);
     a.chunk = a.pc + a.vc < kChunkMax ? a.pc + a.vc : kChunkMax;
-    err = cluster_capacity(C, a.chunk, &cap);
+    smem = kFixedSmem + (size_t)PM * (a.chunk + 2) * sizeof(float2);
+    if (smem < kOwnSmSmem) smem = kOwnSmSmem;
+    err = cluster_capacity(C, smem, &cap);
     if (err != cudaSuccess) return err;
     if (cap >= pairs || C == 1) break;
   }
@@ -700,8 +747,7 @@ cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const d
   const int ncl = pairs < cap ? pairs : cap;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[2];
-  launch_config(&cfg, at, ncl * C, C, kFixedSmem + (size_t)PM * (a.chunk + 2) * sizeof(float2), st,
-                true);
+  launch_config(&cfg, at, ncl * C, C, smem, st, true);
   count_launches(1);
   err = cudaLaunchKernelEx(&cfg, k_jacobi32, a, s.ctl);
   if (err != cudaSuccess) return err;
