@@ -184,28 +184,70 @@ __global__ void k_site_op(const cplx* O, const cplx* K, cplx* Kout, int chl, int
 // ------------------------------------------------------------------ mixing
 constexpr int MIX_MAX = 128;   // largest row/column count of a mixing matrix
 
-__global__ void k_mix(MixPlan pl, MixStrides s, int P, int Q, const cplx* in, long long iP,
-                      long long iQ, cplx* out, long long oP, long long oQ) {
+constexpr int MIX_NNZ = 1024;  // entries staged in shared memory
+constexpr int MIX_Q = 32;      // values of q per block
+constexpr int MIX_G = 8;       // row groups per block
+
+// One block per (p, 32 values of q): thread (q, g) forms the rows g, g + 8, ...
+// The entries (value and input offset) are staged in shared memory, so that a
+// term costs one load of the input and its products; real entries (every spin
+// or fermion operator in use) take two FP64 products per term instead of four.
+// (One thread for all rows of a (p, q), reading the entries from global memory
+// one after the other, took 20-23 us at every size: 32 blocks and a chain of
+// dependent loads at chi = 64, the FP64 pipe at chi = 256.)
+__global__ void __launch_bounds__(MIX_Q* MIX_G)
+k_mix(MixPlan pl, MixStrides s, int P, int Q, const cplx* in, long long iP, long long iQ, cplx* out,
+      long long oP, long long oQ) {
   __shared__ long long ioff[MIX_MAX], ooff[MIX_MAX];
-  for (int j = threadIdx.x; j < pl.ncols; j += blockDim.x) {
+  __shared__ int rp[MIX_MAX + 1];
+  __shared__ long long soff[MIX_NNZ];
+  __shared__ cplx sval[MIX_NNZ];
+  const int tid = threadIdx.x;
+  for (int j = tid; j < pl.ncols; j += blockDim.x) {
     const int j2 = j % pl.cdim[2], j1 = (j / pl.cdim[2]) % pl.cdim[1], j0 = j / (pl.cdim[2] * pl.cdim[1]);
     ioff[j] = j0 * s.ic[0] + j1 * s.ic[1] + j2 * s.ic[2];
   }
-  for (int k = threadIdx.x; k < pl.nrows; k += blockDim.x) {
+  for (int k = tid; k < pl.nrows; k += blockDim.x) {
     const int k2 = k % pl.rdim[2], k1 = (k / pl.rdim[2]) % pl.rdim[1], k0 = k / (pl.rdim[2] * pl.rdim[1]);
     ooff[k] = k0 * s.oc[0] + k1 * s.oc[1] + k2 * s.oc[2];
   }
+  for (int k = tid; k <= pl.nrows; k += blockDim.x) rp[k] = pl.row_ptr[k];
   __syncthreads();
-  const long long tot = (long long)P * Q;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
-       e += (long long)gridDim.x * blockDim.x) {
-    const long long p = e / Q, q = e - p * Q;
+  const bool staged = pl.nnz <= MIX_NNZ;
+  int real = staged;
+  if (staged)
+    for (int e = tid; e < pl.nnz; e += blockDim.x) {
+      const cplx v = pl.val[e];
+      sval[e] = v;
+      soff[e] = ioff[pl.col[e]];
+      if (v.y != 0.0) real = 0;
+    }
+  real = __syncthreads_and(real);
+  const int qt = (Q + MIX_Q - 1) / MIX_Q;
+  const long long tiles = (long long)P * qt;
+  const int ql = tid % MIX_Q, g = tid / MIX_Q;
+  for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    const long long p = t / qt, q = (t - p * qt) * MIX_Q + ql;
+    if (q >= Q) continue;
     const cplx* ib = in + p * iP + q * iQ;
     cplx* ob = out + p * oP + q * oQ;
-    for (int k = 0; k < pl.nrows; ++k) {
+    for (int k = g; k < pl.nrows; k += MIX_G) {
       cplx acc = cmake(0.0, 0.0);
-      for (int t = __ldg(pl.row_ptr + k); t < __ldg(pl.row_ptr + k + 1); ++t)
-        cfma(acc, pl.val[t], ib[ioff[__ldg(pl.col + t)]]);
+      const int e1 = rp[k + 1];
+      if (real) {
+#pragma unroll 4
+        for (int e = rp[k]; e < e1; ++e) {
+          const double v = sval[e].x;
+          const cplx x = ib[soff[e]];
+          acc.x = fma(v, x.x, acc.x);
+          acc.y = fma(v, x.y, acc.y);
+        }
+      } else if (staged) {
+#pragma unroll 4
+        for (int e = rp[k]; e < e1; ++e) cfma(acc, sval[e], ib[soff[e]]);
+      } else {
+        for (int e = rp[k]; e < e1; ++e) cfma(acc, pl.val[e], ib[ioff[__ldg(pl.col + e)]]);
+      }
       ob[ooff[k]] = acc;
     }
   }
@@ -398,10 +440,10 @@ cudaError_t mix_apply(const MixPlan& plan, const MixStrides& s, int P, int Q, co
   if (plan.nrows > MIX_MAX || plan.ncols > MIX_MAX) return cudaErrorInvalidValue;
   const long long tot = (long long)P * Q;
   if (tot <= 0) return cudaSuccess;
-  long long g = (tot + 127) / 128;
-  if (g > 1216) g = 1216;
+  long long g = (long long)P * ((Q + MIX_Q - 1) / MIX_Q);
+  if (g > 152 * 8) g = 152 * 8;
   count_launches(1);
-  k_mix<<<(int)g, 128, 0, st>>>(plan, s, P, Q, in, iP, iQ, out, oP, oQ);
+  k_mix<<<(int)g, MIX_Q * MIX_G, 0, st>>>(plan, s, P, Q, in, iP, iQ, out, oP, oQ);
   return cudaGetLastError();
 }
 cudaError_t gmres_start(GmresState* s, const double* r0norm2, const double* bnorm2,
