@@ -145,9 +145,6 @@ cudaError_t vec_copy(cplx* y, const cplx* x, long long n, cudaStream_t st);
 cudaError_t vec_zero(cplx* y, long long n, cudaStream_t st);
 // y = a*x + b*y  (a, b complex scalars given on the host)
 cudaError_t vec_axpby(cplx* y, const cplx* x, cplx a, cplx b, long long n, cudaStream_t st);
-// out[i] = sum_e conj(V[i*ldv + e]) * w[e], i < nv  (device output); skips if *active == 0
-cudaError_t vec_block_dot(const cplx* V, long long ldv, int nv, const cplx* w, long long n,
-                          cplx* out, cplx* partial, const int* active, cudaStream_t st);
 // w += sign * sum_i h[i] * V[i*ldv + .]  (h on device); skips if *active == 0
 // (if nv_dev is given, only the first min(nv, *nv_dev) vectors are used)
 cudaError_t vec_block_axpy(const cplx* V, long long ldv, int nv, const int* nv_dev,
@@ -177,18 +174,19 @@ struct GmresState {
   double beta, bnorm, wnorm2, inv_h, res;
   int steps, active, breakdown;
 };
-// r0 = B - AX0 is in V0 with |r0|^2 in *norm2: set beta, scale factor, g.
-cudaError_t gmres_start(GmresState* s, const double* r0norm2, const double* bnorm2,
-                        cudaStream_t st);
-// after Arnoldi step j (h1, h2 in s->h, |w|^2 in s->wnorm2): Givens update,
-// breakdown/convergence test, 1/h_{j+1,j} for the next basis vector.
-cudaError_t gmres_step(GmresState* s, int j, int m, double breakdown_rel, double local_tol,
-                       cudaStream_t st);
+// r holds A X0: r = B - r, and the start of a cycle (beta, |B|, 1/beta for the
+// scaling of r, g).  partial: 608 x 32 complex of scratch; counter: a device
+// word that is zero between calls.
+cudaError_t arnoldi_start(cplx* r, const cplx* B, long long n, GmresState* s, cplx* partial,
+                          unsigned int* counter, cudaStream_t st);
+// Arnoldi step j: w (= A v_j) is made orthogonal to V_0..V_j (classical
+// Gram-Schmidt twice), then the Givens update, breakdown/convergence test and
+// 1/h_{j+1,j} for the scaling of w.  Nothing if s->active is 0.
+cudaError_t arnoldi_step(const cplx* V, long long ldv, int j, int m, cplx* w, long long n,
+                         double breakdown_rel, double local_tol, GmresState* s, cplx* partial,
+                         unsigned int* counter, cudaStream_t st);
 // solve the triangular system for y (k = s->steps) and write y into s->y
 cudaError_t gmres_finish(GmresState* s, cudaStream_t st);
-// add the projections of the two Gram-Schmidt passes into column j of H
-cudaError_t gmres_collect(GmresState* s, int j, int m, const cplx* h1, const cplx* h2,
-                          cudaStream_t st);
 
 // ---------------------------------------------------------------- SVD (FP64)
 // Householder LQ of the rows of W (p x q, row-major), in place: row j keeps

@@ -533,7 +533,8 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
   double* nref = wts + k;
   int* perm = reinterpret_cast<int*>(nref + k);
   int* stamps = perm + k;
-  // dcounter words: 8-10 GEMM error flags, 16-39 Jacobi state, 40-47 LQ state
+  // dcounter words: 8-10 GEMM error flags, 16-39 Jacobi state, 40-47 LQ state,
+  // 48 the Krylov reductions' block counter
   unsigned int* jstate = reinterpret_cast<unsigned int*>(ctx->dcounter) + 16;
   unsigned int* lqstate = reinterpret_cast<unsigned int*>(ctx->dcounter) + 40;
   double* anorm2 = ctx->dscal + 8;
@@ -639,27 +640,18 @@ ite_status gmres_cycle(ite_ctx ctx, ite_mpo H, int i, int chl, int chr, const cp
   cplx* V = P<cplx>(ctx->ws_V);
   GmresState* gs = ctx->gm;
   int* active = &gs->active;
-  double* r0n2 = ctx->dscal + 0;
-  double* bn2 = ctx->dscal + 1;
+  unsigned int* counter = reinterpret_cast<unsigned int*>(ctx->dcounter) + 48;
   const cplx ca = alpha, cc = c;
   // r0 = B - A X0
   CS(apply_heff(ctx, H, i, chl, chr, L, R, X, V, cc, X, ca));
-  CK(vec_axpby(V, B, C(1), C(-1), n, ctx->stream));
-  CK(vec_norm2(V, n, r0n2, ctx->dscal + 16, nullptr, ctx->stream));
-  CK(vec_norm2(B, n, bn2, ctx->dscal + 16, nullptr, ctx->stream));
-  CK(gmres_start(gs, r0n2, bn2, ctx->stream));
+  CK(arnoldi_start(V, B, n, gs, ctx->partial, counter, ctx->stream));
   CK(vec_scale_dev(V, &gs->inv_h, n, active, ctx->stream));
   for (int j = 0; j < m; ++j) {
     cplx* vj = V + j * n;
     cplx* w = V + (j + 1) * n;
     CS(apply_heff(ctx, H, i, chl, chr, L, R, vj, w, cc, vj, ca));
-    CK(vec_block_dot(V, n, j + 1, w, n, gs->h, ctx->partial, active, ctx->stream));
-    CK(vec_block_axpy(V, n, j + 1, nullptr, gs->h, -1.0, w, n, active, ctx->stream));
-    CK(vec_block_dot(V, n, j + 1, w, n, gs->h + 32, ctx->partial, active, ctx->stream));
-    CK(vec_block_axpy(V, n, j + 1, nullptr, gs->h + 32, -1.0, w, n, active, ctx->stream));
-    CK(gmres_collect(gs, j, m, gs->h, gs->h + 32, ctx->stream));
-    CK(vec_norm2(w, n, &gs->wnorm2, ctx->dscal + 16, active, ctx->stream));
-    CK(gmres_step(gs, j, m, kBreakdownRel, local_tol, ctx->stream));
+    CK(arnoldi_step(V, n, j, m, w, n, kBreakdownRel, local_tol, gs, ctx->partial, counter,
+                    ctx->stream));
     CK(vec_scale_dev(w, &gs->inv_h, n, active, ctx->stream));
   }
   CK(gmres_finish(gs, ctx->stream));

@@ -1,4 +1,4 @@
-// Krylov vector kernels (block dot, block axpy, norms, scaling), the MPO
+// Krylov vector kernels (Arnoldi step, block axpy, norms, scaling), the MPO
 // mixing kernel, small trace/site-operator kernels and the device-side GMRES
 // control (Givens QR of the Hessenberg matrix) of the local solves.
 //
@@ -54,31 +54,6 @@ __global__ void k_zero(cplx* y, long long n) {
 __global__ void k_axpby(cplx* y, const cplx* x, cplx a, cplx b, long long n) {
   for (long long e = blockIdx.x * (long long)VT + threadIdx.x; e < n; e += (long long)gridDim.x * VT)
     y[e] = cadd(cmul(a, x[e]), cmul(b, y[e]));
-}
-
-// partial[blk*nv + i] = block's share of sum_e conj(V_i[e]) w[e]
-__global__ void k_block_dot(const cplx* V, long long ldv, int nv, const cplx* w, long long n,
-                            cplx* partial, const int* active) {
-  if (active && *active == 0) return;
-  __shared__ double sh[32];
-  for (int i0 = 0; i0 < nv; i0 += 4) {
-    cplx acc[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) acc[u] = cmake(0.0, 0.0);
-    for (long long e = blockIdx.x * (long long)VT + threadIdx.x; e < n; e += (long long)gridDim.x * VT) {
-      const cplx we = w[e];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (i0 + u < nv) cfma_conj(acc[u], V[(long long)(i0 + u) * ldv + e], we);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (i0 + u >= nv) break;
-      const double re = block_sum(acc[u].x, sh);
-      const double im = block_sum(acc[u].y, sh);
-      if (threadIdx.x == 0) partial[(long long)blockIdx.x * nv + i0 + u] = cmake(re, im);
-    }
-  }
 }
 
 // out[i] = sum over the nblk partial rows of column i: warp i takes column
@@ -253,19 +228,195 @@ k_mix(MixPlan pl, MixStrides s, int P, int Q, const cplx* in, long long iP, long
   }
 }
 
-// ------------------------------------------------------------------ GMRES control
+// ------------------------------------------------------------------ Arnoldi step
+// One Arnoldi step of the local solve's GMRES (classical Gram-Schmidt twice) in
+// three kernels and a scaling:
+//   k_arnoldi_dot   h1 = V^H w
+//   k_arnoldi_mid   w -= V h1, h2 = V^H w
+//   k_arnoldi_end   w -= V h2, |w|^2, then the Givens update of the step
+// Each sum ends in the block that finishes last (a counter in device memory),
+// which adds the other blocks' shares in a fixed order, so no kernel is launched
+// to add up 600 numbers; w is read and written by the same thread throughout.
+// Bound: the launches and the FP64 adds of the reductions.  A warp-wide sum of
+// one double takes five adds of 16 clocks on the SM's FP64 pipe, so eight sums
+// are reduced together, halving what a lane holds at each exchange (9 adds
+// instead of 40).  Eleven kernels per step before (n = 16384, chi = 64: 13 us a
+// dot, 12 us for the Givens update by one thread reading global memory); now
+// 9.6, 10.8 and 17 us for the three at chi = 64, the last 10 of them the chain of
+// the Givens update.  GMRES(10): 1.91 -> 1.56 ms at chi = 64.
+constexpr int AT = 128;          // threads per block
+constexpr int AW = AT / 32;
+
+int arnoldi_grid(long long n) {
+  long long g = (n + AT - 1) / AT;
+  return (int)(g > 608 ? 608 : g < 1 ? 1 : g);
+}
+
+// Sums v[0..8) over the warp; the lanes with lane % 4 == 0 return sum number
+// (lane >> 2) (bits 4, 3, 2 of the lane select the half kept at each exchange).
+__device__ __forceinline__ double warp_sum8(double (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int n = 4, m = 16; n >= 1; n >>= 1, m >>= 1) {
+    const bool up = (lane & m) != 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const double send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+    }
+  }
+  double r = v[0];
+  r += __shfl_xor_sync(0xffffffffu, r, 2);
+  r += __shfl_xor_sync(0xffffffffu, r, 1);
+  return r;
+}
+
+// sh[warp][2 i], sh[warp][2 i + 1] = this warp's share of conj(V_i) . w over the
+// elements of its threads
+__device__ __forceinline__ void dot_shares(const cplx* V, long long ldv, int nv, const cplx* w,
+                                           long long n, double (*sh)[2 * MAXV + 6]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int i0 = 0; i0 < nv; i0 += 4) {
+    cplx acc[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) acc[u] = cmake(0.0, 0.0);
+    for (long long e = blockIdx.x * (long long)AT + threadIdx.x; e < n; e += (long long)gridDim.x * AT) {
+      const cplx we = w[e];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i0 + u < nv) cfma_conj(acc[u], V[(long long)(i0 + u) * ldv + e], we);
+    }
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      v[2 * u] = acc[u].x;
+      v[2 * u + 1] = acc[u].y;
+    }
+    const double r = warp_sum8(v);
+    if ((lane & 3) == 0) sh[wid][2 * i0 + (lane >> 2)] = r;
+  }
+}
+
+// w -= sum_i h_i V_i on the elements of this thread; h in shared memory
+__device__ __forceinline__ void subtract(const cplx* V, long long ldv, int nv, const cplx* hs,
+                                         cplx* w, long long n) {
+  for (long long e = blockIdx.x * (long long)AT + threadIdx.x; e < n; e += (long long)gridDim.x * AT) {
+    cplx acc = w[e];
+    for (int i = 0; i < nv; ++i) cfma(acc, hs[i], V[(long long)i * ldv + e]);
+    w[e] = acc;
+  }
+}
+
+// True in the block that arrives last, which then sees what the others wrote
+// before they arrived; leaves the counter at zero.
+__device__ __forceinline__ bool last_block(unsigned int* counter) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    if (last) *counter = 0u;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// The block's shares to `partial` (2 nv doubles per block), and in the last block
+// the sums, in block order, to out
+__device__ __forceinline__ void finish_dots(int nv, double (*sh)[2 * MAXV + 6], cplx* partial,
+                                            cplx* out, unsigned int* counter) {
+  __syncthreads();
+  double* p = reinterpret_cast<double*>(partial);
+  for (int c = threadIdx.x; c < 2 * nv; c += AT) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < AW; ++w) t += sh[w][c];
+    p[(long long)blockIdx.x * 2 * nv + c] = t;
+  }
+  if (!last_block(counter)) return;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int i = wid; i < nv; i += AW) {
+    double sr = 0.0, si = 0.0;
+    for (unsigned int b = lane; b < gridDim.x; b += 32) {
+      const cplx v = __ldcg(partial + (long long)b * nv + i);
+      sr += v.x;
+      si += v.y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      sr += __shfl_xor_sync(0xffffffffu, sr, o);
+      si += __shfl_xor_sync(0xffffffffu, si, o);
+    }
+    if (lane == 0) out[i] = cmake(sr, si);
+  }
+}
+
+// Two real sums over the block (valid in thread 0)
+__device__ __forceinline__ void block_sum_pair(double& a, double& b) {
+  __shared__ double sh[AW][2];
+  a = warp_sum(a);
+  b = warp_sum(b);
+  if ((threadIdx.x & 31) == 0) {
+    sh[threadIdx.x >> 5][0] = a;
+    sh[threadIdx.x >> 5][1] = b;
+  }
+  __syncthreads();
+  a = b = 0.0;
+#pragma unroll
+  for (int w = 0; w < AW; ++w) {
+    a += sh[w][0];
+    b += sh[w][1];
+  }
+}
+
+// Sums over all blocks' (a, b) in the last block, in every lane of its first
+// warp; returns false in all other threads
+__device__ __forceinline__ bool total_pair(double& a, double& b, cplx* partial,
+                                           unsigned int* counter) {
+  if (threadIdx.x == 0) partial[blockIdx.x] = cmake(a, b);
+  if (!last_block(counter) || threadIdx.x >= 32) return false;
+  a = b = 0.0;
+  for (unsigned int k = threadIdx.x; k < gridDim.x; k += 32) {
+    const cplx v = __ldcg(partial + k);
+    a += v.x;
+    b += v.y;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  return true;
+}
+
 __device__ __forceinline__ cplx& Hc(GmresState* s, int i, int j) { return s->H[j * (32 + 1) + i]; }
 
-__global__ void k_gmres_start(GmresState* s, const double* r0n2, const double* bn2) {
-  const double beta = sqrt(*r0n2);
+// r = B - r, |r|^2 and |B|^2, and the start of the cycle
+__global__ void __launch_bounds__(AT)
+k_arnoldi_start(cplx* r, const cplx* B, long long n, GmresState* s, cplx* partial,
+                unsigned int* counter) {
+  double a = 0.0, b = 0.0;
+  for (long long e = blockIdx.x * (long long)AT + threadIdx.x; e < n; e += (long long)gridDim.x * AT) {
+    const cplx be = B[e], v = csub(be, r[e]);
+    r[e] = v;
+    a = fma(v.x, v.x, fma(v.y, v.y, a));
+    b = fma(be.x, be.x, fma(be.y, be.y, b));
+  }
+  block_sum_pair(a, b);
+  if (!total_pair(a, b, partial, counter)) return;
+  const int lane = threadIdx.x;
+  for (int i = lane; i < 33; i += 32) s->g[i] = cmake(0.0, 0.0);
+  s->y[lane] = cmake(0.0, 0.0);
+  for (int i = lane; i < 33 * 32; i += 32) s->H[i] = cmake(0.0, 0.0);
+  __syncwarp();
+  if (lane != 0) return;
+  const double beta = sqrt(a);
   s->beta = beta;
-  s->bnorm = sqrt(*bn2);
+  s->bnorm = sqrt(b);
   s->steps = 0;
   s->breakdown = 0;
   s->res = beta;
-  for (int i = 0; i < 33; ++i) s->g[i] = cmake(0.0, 0.0);
-  for (int i = 0; i < 32; ++i) s->y[i] = cmake(0.0, 0.0);
-  for (int i = 0; i < 33 * 32; ++i) s->H[i] = cmake(0.0, 0.0);
   if (beta > 0.0 && isfinite(beta)) {
     s->active = 1;
     s->inv_h = 1.0 / beta;
@@ -276,72 +427,140 @@ __global__ void k_gmres_start(GmresState* s, const double* r0n2, const double* b
   }
 }
 
-__global__ void k_gmres_collect(GmresState* s, int j, const cplx* h1, const cplx* h2) {
-  if (!s->active) return;
-  const int i = threadIdx.x;
-  if (i <= j) Hc(s, i, j) = cadd(h1[i], h2[i]);
+__global__ void __launch_bounds__(AT)
+k_arnoldi_dot(const cplx* V, long long ldv, int nv, const cplx* w, long long n, GmresState* s,
+              cplx* partial, unsigned int* counter) {
+  if (s->active == 0) return;
+  __shared__ double sh[AW][2 * MAXV + 6];
+  dot_shares(V, ldv, nv, w, n, sh);
+  finish_dots(nv, sh, partial, s->h, counter);
 }
 
-__global__ void k_gmres_step(GmresState* s, int j, int m, double brel, double ltol) {
-  if (!s->active) return;
-  const double hj1 = sqrt(s->wnorm2);
-  // |A v_j|^2 = sum_i |h_ij|^2 + h_{j+1,j}^2 (Arnoldi relation), read before
-  // the rotations touch column j; a happy breakdown is a new direction that
-  // is negligible against it
-  double col2 = s->wnorm2;
-  for (int i = 0; i <= j; ++i) {
-    const cplx h = Hc(s, i, j);
-    col2 = fma(h.x, h.x, fma(h.y, h.y, col2));
-  }
-  // earlier rotations on column j
-  for (int i = 0; i < j; ++i) {
-    const cplx a = Hc(s, i, j), b = Hc(s, i + 1, j);
-    const cplx c = s->cs[i], sn = s->sn[i];
-    Hc(s, i, j) = cadd(cmul(c, a), cmul(sn, b));
-    Hc(s, i + 1, j) = csub(cmul(c, b), cmul(cconj(sn), a));
-  }
-  // new rotation zeroing h_{j+1,j}
-  const cplx a = Hc(s, j, j);
-  const double an = hypot(a.x, a.y);
-  const double r = hypot(an, hj1);
-  cplx c, sn;
-  if (r == 0.0) {
-    c = cmake(1.0, 0.0); sn = cmake(0.0, 0.0);
-  } else if (an == 0.0) {
-    c = cmake(0.0, 0.0); sn = cmake(1.0, 0.0);
-  } else {
-    c = cmake(an / r, 0.0);
-    sn = cscale(a, hj1 / (an * r));
-  }
-  s->cs[j] = c;
-  s->sn[j] = sn;
-  Hc(s, j, j) = (an == 0.0) ? cmake(hj1, 0.0) : cscale(a, r / an);
-  Hc(s, j + 1, j) = cmake(0.0, 0.0);
-  const cplx gj = s->g[j];
-  s->g[j] = cmul(c, gj);
-  s->g[j + 1] = cscale(cmul(cconj(sn), gj), -1.0);
-  s->res = hypot(s->g[j + 1].x, s->g[j + 1].y);
-  s->steps = j + 1;
-  if (!(hj1 > brel * sqrt(col2)) || !isfinite(hj1)) {
-    s->breakdown = 1;
-    s->active = 0;
-  } else if (ltol > 0.0 && s->res <= ltol * s->bnorm) {
-    s->active = 0;
-  } else if (j + 1 >= m) {
-    s->active = 0;
-  } else {
-    s->inv_h = 1.0 / hj1;
-  }
+__global__ void __launch_bounds__(AT)
+k_arnoldi_mid(const cplx* V, long long ldv, int nv, cplx* w, long long n, GmresState* s,
+              cplx* partial, unsigned int* counter) {
+  if (s->active == 0) return;
+  __shared__ double sh[AW][2 * MAXV + 6];
+  __shared__ cplx hs[MAXV];
+  for (int i = threadIdx.x; i < nv; i += AT) hs[i] = cscale(s->h[i], -1.0);
+  __syncthreads();
+  subtract(V, ldv, nv, hs, w, n);
+  dot_shares(V, ldv, nv, w, n, sh);
+  finish_dots(nv, sh, partial, s->h + 32, counter);
 }
 
-__global__ void k_gmres_finish(GmresState* s) {
-  const int k = s->steps;
+// Column j of H from the two passes' projections and |w|^2, the Givens update
+// and the tests that end the cycle (one warp: the column and the earlier
+// rotations are fetched together, the chain of rotations runs in lane 0).
+__device__ void gmres_step(GmresState* s, int j, int m, double brel, double ltol, double wnorm2,
+                           cplx* col, cplx* cs, cplx* sn) {
+  const int lane = threadIdx.x;
+  double c2 = 0.0;
+  if (lane <= j) {
+    const cplx h = cadd(s->h[lane], s->h[32 + lane]);
+    col[lane] = h;
+    c2 = fma(h.x, h.x, h.y * h.y);
+    if (lane < j) {
+      cs[lane] = s->cs[lane];
+      sn[lane] = s->sn[lane];
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) c2 += __shfl_xor_sync(0xffffffffu, c2, o);
+  __syncwarp();
+  if (lane == 0) {
+    s->wnorm2 = wnorm2;
+    const double hj1 = sqrt(wnorm2);
+    // |A v_j|^2 = sum_i |h_ij|^2 + h_{j+1,j}^2 (Arnoldi relation); a happy
+    // breakdown is a new direction that is negligible against it
+    const double col2 = wnorm2 + c2;
+    cplx a = col[0];
+    for (int i = 0; i < j; ++i) {
+      const cplx b = col[i + 1], c = cs[i], t = sn[i];
+      col[i] = cadd(cmul(c, a), cmul(t, b));
+      a = csub(cmul(c, b), cmul(cconj(t), a));
+    }
+    // new rotation zeroing h_{j+1,j}
+    const double an = hypot(a.x, a.y);
+    const double r = hypot(an, hj1);
+    cplx c, t;
+    if (r == 0.0) {
+      c = cmake(1.0, 0.0); t = cmake(0.0, 0.0);
+    } else if (an == 0.0) {
+      c = cmake(0.0, 0.0); t = cmake(1.0, 0.0);
+    } else {
+      c = cmake(an / r, 0.0);
+      t = cscale(a, hj1 / (an * r));
+    }
+    s->cs[j] = c;
+    s->sn[j] = t;
+    col[j] = (an == 0.0) ? cmake(hj1, 0.0) : cscale(a, r / an);
+    const cplx gj = s->g[j];
+    const cplx g1 = cscale(cmul(cconj(t), gj), -1.0);
+    s->g[j] = cmul(c, gj);
+    s->g[j + 1] = g1;
+    const double res = hypot(g1.x, g1.y);
+    s->res = res;
+    s->steps = j + 1;
+    if (!(hj1 > brel * sqrt(col2)) || !isfinite(hj1)) {
+      s->breakdown = 1;
+      s->active = 0;
+    } else if (ltol > 0.0 && res <= ltol * s->bnorm) {
+      s->active = 0;
+    } else if (j + 1 >= m) {
+      s->active = 0;
+    } else {
+      s->inv_h = 1.0 / hj1;
+    }
+  }
+  __syncwarp();
+  if (lane <= j) Hc(s, lane, j) = col[lane];
+}
+
+__global__ void __launch_bounds__(AT)
+k_arnoldi_end(const cplx* V, long long ldv, int j, int m, cplx* w, long long n, double brel,
+              double ltol, GmresState* s, cplx* partial, unsigned int* counter) {
+  if (s->active == 0) return;
+  __shared__ cplx hs[MAXV], cs[MAXV], sn[MAXV];
+  for (int i = threadIdx.x; i <= j; i += AT) hs[i] = cscale(s->h[32 + i], -1.0);
+  __syncthreads();
+  double a = 0.0, b = 0.0;
+  for (long long e = blockIdx.x * (long long)AT + threadIdx.x; e < n; e += (long long)gridDim.x * AT) {
+    cplx acc = w[e];
+    for (int i = 0; i <= j; ++i) cfma(acc, hs[i], V[(long long)i * ldv + e]);
+    w[e] = acc;
+    a = fma(acc.x, acc.x, fma(acc.y, acc.y, a));
+  }
+  block_sum_pair(a, b);
+  if (!total_pair(a, b, partial, counter)) return;
+  gmres_step(s, j, m, brel, ltol, a, hs, cs, sn);
+}
+
+// y of the triangular system (one warp; row i's products by the lanes)
+__global__ void __launch_bounds__(32) k_gmres_finish(GmresState* s) {
+  __shared__ cplx y[MAXV];
+  const int k = s->steps, lane = threadIdx.x;
   for (int i = k - 1; i >= 0; --i) {
-    cplx acc = s->g[i];
-    for (int l = i + 1; l < k; ++l) acc = csub(acc, cmul(Hc(s, i, l), s->y[l]));
-    const cplx d = Hc(s, i, i);
-    const double dn = d.x * d.x + d.y * d.y;
-    s->y[i] = (dn > 0.0) ? cscale(cmul(acc, cconj(d)), 1.0 / dn) : cmake(0.0, 0.0);
+    const int l = i + 1 + lane;
+    double sr = 0.0, si = 0.0;
+    if (l < k) {
+      const cplx t = cmul(Hc(s, i, l), y[l]);
+      sr = t.x;
+      si = t.y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      sr += __shfl_xor_sync(0xffffffffu, sr, o);
+      si += __shfl_xor_sync(0xffffffffu, si, o);
+    }
+    if (lane == 0) {
+      const cplx acc = csub(s->g[i], cmake(sr, si)), d = Hc(s, i, i);
+      const double dn = d.x * d.x + d.y * d.y;
+      const cplx v = (dn > 0.0) ? cscale(cmul(acc, cconj(d)), 1.0 / dn) : cmake(0.0, 0.0);
+      y[i] = v;
+      s->y[i] = v;
+    }
+    __syncwarp();
   }
 }
 
@@ -363,17 +582,6 @@ cudaError_t vec_axpby(cplx* y, const cplx* x, cplx a, cplx b, long long n, cudaS
   if (n <= 0) return cudaSuccess;
   count_launches(1);
   k_axpby<<<grid_for(n), VT, 0, st>>>(y, x, a, b, n);
-  return cudaGetLastError();
-}
-cudaError_t vec_block_dot(const cplx* V, long long ldv, int nv, const cplx* w, long long n,
-                          cplx* out, cplx* partial, const int* active, cudaStream_t st) {
-  if (nv <= 0) return cudaSuccess;
-  if (nv > MAXV) return cudaErrorInvalidValue;
-  const int g = grid_for(n);
-  count_launches(1);
-  k_block_dot<<<g, VT, 0, st>>>(V, ldv, nv, w, n, partial, active);
-  count_launches(1);
-  k_reduce_cplx<<<1, 32 * nv, 0, st>>>(partial, g, nv, out, active);
   return cudaGetLastError();
 }
 cudaError_t vec_block_axpy(const cplx* V, long long ldv, int nv, const int* nv_dev,
@@ -446,28 +654,26 @@ cudaError_t mix_apply(const MixPlan& plan, const MixStrides& s, int P, int Q, co
   k_mix<<<(int)g, MIX_Q * MIX_G, 0, st>>>(plan, s, P, Q, in, iP, iQ, out, oP, oQ);
   return cudaGetLastError();
 }
-cudaError_t gmres_start(GmresState* s, const double* r0norm2, const double* bnorm2,
-                        cudaStream_t st) {
+cudaError_t arnoldi_start(cplx* r, const cplx* B, long long n, GmresState* s, cplx* partial,
+                          unsigned int* counter, cudaStream_t st) {
   count_launches(1);
-  k_gmres_start<<<1, 1, 0, st>>>(s, r0norm2, bnorm2);
+  k_arnoldi_start<<<arnoldi_grid(n), AT, 0, st>>>(r, B, n, s, partial, counter);
   return cudaGetLastError();
 }
-cudaError_t gmres_collect(GmresState* s, int j, int m, const cplx* h1, const cplx* h2,
-                          cudaStream_t st) {
-  (void)m;
-  count_launches(1);
-  k_gmres_collect<<<1, 32, 0, st>>>(s, j, h1, h2);
-  return cudaGetLastError();
-}
-cudaError_t gmres_step(GmresState* s, int j, int m, double breakdown_rel, double local_tol,
-                       cudaStream_t st) {
-  count_launches(1);
-  k_gmres_step<<<1, 1, 0, st>>>(s, j, m, breakdown_rel, local_tol);
+cudaError_t arnoldi_step(const cplx* V, long long ldv, int j, int m, cplx* w, long long n,
+                         double breakdown_rel, double local_tol, GmresState* s, cplx* partial,
+                         unsigned int* counter, cudaStream_t st) {
+  if (j < 0 || j >= MAXV || n <= 0) return cudaErrorInvalidValue;
+  const int g = arnoldi_grid(n);
+  count_launches(3);
+  k_arnoldi_dot<<<g, AT, 0, st>>>(V, ldv, j + 1, w, n, s, partial, counter);
+  k_arnoldi_mid<<<g, AT, 0, st>>>(V, ldv, j + 1, w, n, s, partial, counter);
+  k_arnoldi_end<<<g, AT, 0, st>>>(V, ldv, j, m, w, n, breakdown_rel, local_tol, s, partial, counter);
   return cudaGetLastError();
 }
 cudaError_t gmres_finish(GmresState* s, cudaStream_t st) {
   count_launches(1);
-  k_gmres_finish<<<1, 1, 0, st>>>(s);
+  k_gmres_finish<<<1, 32, 0, st>>>(s);
   return cudaGetLastError();
 }
 
