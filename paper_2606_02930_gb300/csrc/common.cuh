@@ -194,9 +194,9 @@ cudaError_t gmres_finish(GmresState* s, cudaStream_t st);
 // One cooperative launch; dev_state (8 device words) gets a nonzero word 4 if
 // a grid-barrier wait ran out.
 // refl (device, 3 k doubles, may be NULL) receives each reflector's
-// (Re u_0, Im u_0, c) for lq_formq.
-cudaError_t svd_lq(cplx* W, int p, int q, cplx* beta, double* refl, unsigned int* dev_state,
-                   cudaStream_t st);
+// (Re u_0, Im u_0, c) for lq_formq.  pub (k q complex) is scratch.
+cudaError_t svd_lq(cplx* W, int p, int q, cplx* beta, double* refl, cplx* pub,
+                   unsigned int* dev_state, cudaStream_t st);
 // L (p x k, row-major) with Xr = L Q^H from the output of svd_lq
 cudaError_t lq_left(const cplx* W, const cplx* beta, int p, int q, cplx* Lout, cudaStream_t st);
 // *out = |L1^{-1}|_F^2 for the leading k x k triangle L1 of svd_lq's L (+inf
@@ -205,9 +205,8 @@ cudaError_t lq_left(const cplx* W, const cplx* beta, int p, int q, cplx* Lout, c
 cudaError_t lq_inv_fnorm2(const cplx* W, const cplx* beta, int q, int k, double* colnorm2,
                           double* out, cudaStream_t st);
 // Qh (k x q) = Q^H, the orthonormal rows with Xr = L Q^H, from svd_lq's
-// output and refl.  One cooperative launch; dev_state (8 words) as svd_lq.
-cudaError_t lq_formq(const cplx* W, const double* refl, int q, int k, cplx* Qh,
-                     unsigned int* dev_state, cudaStream_t st);
+// output and refl.
+cudaError_t lq_formq(const cplx* W, const double* refl, int q, int k, cplx* Qh, cudaStream_t st);
 // R (k x p, k = min(p, q)) = L^H from the output of svd_lq
 cudaError_t svd_lq_r(const cplx* W, const cplx* beta, int p, int q, cplx* R, cudaStream_t st);
 // Preconditioner of the Jacobi (svd_pre.cu): its workspace for a k x p factor R

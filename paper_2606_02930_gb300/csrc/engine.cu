@@ -549,7 +549,8 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
     for (int j = 0; j < k; ++j) f += 4.0 * (q - j) + 16.0 * (q - j) * (p - j - 1);
     ctx->lq_flops += f;
     Scope lq_scope(ctx, P_LQ, f);
-    CK(svd_lq(W, p, q, beta, nullptr, lqstate, ctx->stream));
+    CS(buf_ensure(ctx, ctx->ws_V, (size_t)k * q * sizeof(cplx)));
+    CK(svd_lq(W, p, q, beta, nullptr, P<cplx>(ctx->ws_V), lqstate, ctx->stream));
   }
   CK(svd_lq_r(W, beta, p, q, R, ctx->stream));
   // 3. one-sided Jacobi on the k rows (length p) of R, preconditioned where
@@ -956,7 +957,8 @@ ite_status gauge_lq(ite_ctx ctx, const cplx* X, int m, int n, cplx* left, cplx* 
   double* inv2 = ctx->dscal + 10;
   CK(vec_copy(W, X, (long long)m * n, ctx->stream));
   CK(scaled_norm2(W, (long long)m * n, 1.0, anorm2, ctx->dscal + 16, ctx->stream));
-  CK(svd_lq(W, m, n, beta, refl, lqstate, ctx->stream));
+  CS(buf_ensure(ctx, ctx->ws_V, (size_t)k * n * sizeof(cplx)));
+  CK(svd_lq(W, m, n, beta, refl, P<cplx>(ctx->ws_V), lqstate, ctx->stream));
   CK(lq_inv_fnorm2(W, beta, n, k, colnorm, inv2, ctx->stream));
   CK(cudaMemcpyAsync(&ctx->hr->d[2], anorm2, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaMemcpyAsync(&ctx->hr->d[3], inv2, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
@@ -967,7 +969,7 @@ ite_status gauge_lq(ite_ctx ctx, const cplx* X, int m, int n, cplx* left, cplx* 
   if (!(total > 0.0) || !std::isfinite(inv) || !(inv > 0.0) || 1.0 / inv <= kGaugeCertRel * total)
     return ITE_OK;
   CK(lq_left(W, beta, m, n, left, ctx->stream));
-  CK(lq_formq(W, refl, n, k, right, lqstate, ctx->stream));
+  CK(lq_formq(W, refl, n, k, right, ctx->stream));
   *ok = true;
   return ITE_OK;
 }

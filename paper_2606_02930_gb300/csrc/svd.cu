@@ -151,6 +151,236 @@ k_lq_persistent(cplx* W, int p, int q, cplx* beta, double* refl, unsigned int* s
   }
 }
 
+// The same LQ with every row kept in the shared memory of one block (row i in
+// block i mod nb) and the pivot rows handed on through memory without a
+// barrier.  Step j needs nothing but row j: the block that owns row j + 1
+// updates that row first, stores it to `pub`, and then updates its other rows;
+// the others poll pub, which starts as a pattern that is never stored, so the
+// data are their own flag (one trip to L2 between two pivots instead of a
+// store, a fence, a barrier and a load).  Four warps per block, one for each
+// quarter of the SM: a quarter takes 64 clocks per FP64 warp instruction, so what
+// a warp issues one after the other is what a step waits for.  Sums over a warp
+// are taken eight at a time, and the scalars of the reflector by the lanes of
+// one warp side by side.
+// Polls are bounded; a block that gives up sets the error word, which the others
+// see in their own polls, and leaves.
+// Measured, with the barrier kernel above before: 64 x 64 0.41 -> 0.26 ms, 512 x 512
+// 6.4 -> 2.7, 1024 x 1024 25.7 -> 11.6 (5.3 us a step at 512: about 1 us from store
+// to load, the rest the FP64 chain of the next pivot row; at 1024 the seven rows a
+// block holds).
+constexpr int LT = 128;                       // threads
+constexpr int LW = LT / 32;
+constexpr int LC = 3;                         // rows whose inner products are reduced together
+constexpr unsigned long long kUnset = ~0ull;  // pattern of memory that has not been stored to
+
+__device__ __forceinline__ void store_pub(cplx* p, cplx v) {
+  unsigned long long a = (unsigned long long)__double_as_longlong(v.x);
+  unsigned long long b = (unsigned long long)__double_as_longlong(v.y);
+  if (a == kUnset) a = 0x7FF8000000000000ull;   // another NaN
+  if (b == kUnset) b = 0x7FF8000000000000ull;
+  asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
+}
+
+__device__ __forceinline__ bool load_pub(const cplx* p, cplx& v) {
+  unsigned long long a, b;
+  asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+  v = cmake(__longlong_as_double((long long)a), __longlong_as_double((long long)b));
+  return a != kUnset && b != kUnset;
+}
+
+// v[0..8) summed over the warp: the lanes with lane % 4 == 0 return sum lane / 4
+// (half of what a lane holds goes at each exchange: 9 adds instead of 40)
+__device__ __forceinline__ double warp_sum8(double (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int n = 4, m = 16; n >= 1; n >>= 1, m >>= 1) {
+    const bool up = (lane & m) != 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const double send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+    }
+  }
+  double r = v[0];
+  r += __shfl_xor_sync(0xffffffffu, r, 2);
+  r += __shfl_xor_sync(0xffffffffu, r, 1);
+  return r;
+}
+
+constexpr double kTinySq = 1e-280, kHugeSq = 1e280;   // range of the two functions below
+
+// 1 / sqrt(x) and 1 / x for x in that range from the hardware's approximations
+// (about 20 bits) and one step of third order each, e = 1 - x y^2 (or 1 - x y):
+// y (1 + e / 2 + 3 e^2 / 8) and y (1 + e + e^2), to about an ulp.
+__device__ __forceinline__ double rsqrt_fp64(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+__device__ __forceinline__ double rcp_fp64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// One element of a row per thread and LT columns: EPT >= q / LT
+template <int EPT>
+__global__ void __launch_bounds__(LT)
+k_lq_resident(cplx* W, int p, int q, cplx* beta, double* refl, cplx* pub, unsigned int* st) {
+  extern __shared__ cplx rows[];              // local row l, column e: rows[l * EPT * LT + e]
+  __shared__ double sh[LW][8];
+  __shared__ cplx yj[LC], fac[LC];
+  __shared__ cplx s_x0, s_u0, s_du;
+  __shared__ double s_c;
+  __shared__ int s_fail;
+  constexpr int LD = EPT * LT;
+  const int k = p < q ? p : q, nb = (int)gridDim.x, bid = (int)blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int nloc = (p - bid + nb - 1) / nb;   // rows bid, bid + nb, ...
+  if (tid == 0) s_fail = 0;
+  for (int l = 0; l < nloc; ++l)
+    for (int e = tid; e < LD; e += LT)
+      rows[l * LD + e] = e < q ? W[(long long)(bid + l * nb) * q + e] : cmake(0.0, 0.0);
+  if (bid == 0)
+    for (int e = tid; e < q; e += LT) store_pub(pub + e, rows[e]);
+  __syncthreads();
+  for (int j = 0; j < k; ++j) {
+    if (bid + (nloc - 1) * nb < j) break;     // every own row has been a pivot
+    const bool owner = j % nb == bid;
+    // ---- the pivot row's tail (zero left of j)
+    cplx x[EPT];
+    if (owner) {
+#pragma unroll
+      for (int i = 0; i < EPT; ++i) {
+        const int e = tid + LT * i;
+        x[i] = e >= j ? rows[j / nb * LD + e] : cmake(0.0, 0.0);
+      }
+    } else {
+      const cplx* src = pub + (long long)j * q;
+#pragma unroll
+      for (int i = EPT - 1; i >= 0; --i) {
+        const int e = tid + LT * i;
+        x[i] = cmake(0.0, 0.0);
+        if (e >= j && e < q) {
+          bool ok = load_pub(src + e, x[i]);
+          // only the first element of a thread normally has to wait
+          for (unsigned int spins = 0; !ok; ++spins) {
+            if ((spins & 255u) == 255u && *((volatile unsigned int*)(st + 4)) != 0u) break;
+            if (spins > (1u << 23)) {
+              atomicExch(st + 4, 1u);
+              break;
+            }
+            ok = load_pub(src + e, x[i]);
+          }
+          if (!ok) s_fail = 1;
+        }
+      }
+    }
+    // ---- own rows below j; the next pivot first and alone
+    int l = j / nb + (bid <= j % nb ? 1 : 0);
+    bool first = true;
+    while (first || l < nloc) {
+      const bool next = first && bid + l * nb == j + 1;
+      const int nr = min(nloc - l, next ? 1 : LC);
+      cplx* const y = rows + l * LD;
+      double v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = 0.0;
+#pragma unroll
+      for (int i = 0; i < EPT; ++i) {
+        if (LT * (i + 1) <= j) continue;      // columns left of the pivot
+        const int e = tid + LT * i;
+#pragma unroll
+        for (int r = 0; r < LC; ++r)
+          if (r < nr) {
+            const cplx t = y[r * LD + e];     // y conj(x)
+            v[2 * r] = fma(t.x, x[i].x, fma(t.y, x[i].y, v[2 * r]));
+            v[2 * r + 1] = fma(t.y, x[i].x, fma(-t.x, x[i].y, v[2 * r + 1]));
+            if (e == j) yj[r] = t;
+          }
+        if (first) {
+          v[6] = fma(x[i].x, x[i].x, fma(x[i].y, x[i].y, v[6]));
+          if (e == j) s_x0 = x[i];
+        }
+      }
+      const double sum = warp_sum8(v);
+      if ((lane & 3) == 0) sh[w][lane >> 2] = sum;
+      __syncthreads();
+      if (s_fail != 0) return;                // every thread reads the same flag
+      if (w == 0) {
+        // lane v: the block's sum v (6: |x|^2, its lane 7 beside it |x_0|^2)
+        double t = 0.0;
+        if (lane < 7) t = (sh[0][lane] + sh[1][lane]) + (sh[2][lane] + sh[3][lane]);
+        if (first) {
+          // u_0 = x_0 (1 + |x| / |x_0|), c = 1 / (|x|^2 + |x| |x_0|)
+          const cplx x0 = s_x0;
+          if (lane == 7) t = fma(x0.x, x0.x, x0.y * x0.y);
+          double rs = 0.0;
+          if (t > kTinySq && t < kHugeSq) rs = rsqrt_fp64(t);
+          else if (t > 0.0) rs = rsqrt(t);
+          const double n2 = __shfl_sync(0xffffffffu, t, 6);
+          const double a2 = __shfl_sync(0xffffffffu, t, 7), ra = __shfl_sync(0xffffffffu, rs, 7);
+          const double nx = n2 * __shfl_sync(0xffffffffu, rs, 6);
+          const double g = nx * ra;
+          const cplx du = a2 > 0.0 ? cmake(x0.x * g, x0.y * g) : cmake(nx, 0.0);   // u_0 - x_0
+          const double den = fma(nx, a2 * ra, n2);
+          const double c = den > kTinySq && den < kHugeSq ? rcp_fp64(den) : n2 > 0.0 ? 1.0 / den : 0.0;
+          if (lane == 0) {
+            s_c = c;
+            s_du = du;
+            const cplx u0 = cadd(x0, du);
+            s_u0 = u0;
+            if (owner) {
+              beta[j] = cmake(-du.x, -du.y);
+              if (refl) {
+                refl[3 * j] = u0.x;
+                refl[3 * j + 1] = u0.y;
+                refl[3 * j + 2] = c;
+              }
+            }
+          }
+          __syncwarp();
+        }
+        // c (y u^H) of row lane / 2, real and imaginary part in lanes 2 r and
+        // 2 r + 1; the inner product was taken with x_0 instead of u_0
+        if (lane < 2 * nr) {
+          const cplx z = yj[lane >> 1], du = s_du;
+          const bool im = lane & 1;
+          const double f = s_c * fma(im ? z.y : z.x, du.x, fma(im ? -z.x : z.y, du.y, t));
+          reinterpret_cast<double*>(fac)[lane] = f;
+        }
+      }
+      __syncthreads();
+      if (s_c != 0.0) {
+#pragma unroll
+        for (int i = 0; i < EPT; ++i) {
+          if (LT * (i + 1) <= j) continue;
+          const int e = tid + LT * i;
+          const cplx u = e == j ? s_u0 : x[i];
+#pragma unroll
+          for (int r = 0; r < LC; ++r)
+            if (r < nr) {
+              const cplx f = fac[r];
+              cplx t = y[r * LD + e];
+              t.x = fma(-f.x, u.x, fma(f.y, u.y, t.x));
+              t.y = fma(-f.x, u.y, fma(-f.y, u.x, t.y));
+              y[r * LD + e] = t;
+            }
+        }
+      }
+      if (next && j + 1 < k)
+        for (int e = tid; e < q; e += LT)
+          if (e > j) store_pub(pub + (long long)(j + 1) * q + e, y[e]);
+      l += nr;
+      first = false;
+    }
+  }
+  for (int l = 0; l < nloc; ++l)
+    for (int e = tid; e < q; e += LT) W[(long long)(bid + l * nb) * q + e] = rows[l * LD + e];
+}
+
 // R (k x p) = L^H: R[j][i] = conj(L[i][j]); L[i][j] = W[i][j] below the
 // diagonal, beta[j] on it, zero above.
 __global__ void k_lq_r(const cplx* W, const cplx* beta, int p, int q, int k, cplx* R) {
@@ -237,52 +467,120 @@ __global__ void k_sum_small(const double* x, int n, double* out) {
   }
 }
 
-// rows of the k x q identity
-__global__ void k_eye_rows(cplx* Q, int k, int q) {
-  const long long tot = (long long)k * q;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e / q), j = (int)(e - (long long)i * q);
-    Q[e] = cmake(i == j ? 1.0 : 0.0, 0.0);
-  }
-}
-
 // Q^H (k x q, orthonormal rows) with X = L Q^H, from the reflectors of the
 // LQ: the reflectors are Hermitian, so Q^H is the first k rows of
 // H_{k-1} ... H_0, accumulated backwards: starting from identity rows, step
 // j = k-1, ..., 0 applies y <- y - c_j (y u_j^H) u_j to rows j..k-1 (rows
-// above j are still unit vectors that H_j leaves alone).  One grid barrier
-// separates the steps.
+// above j are still unit vectors that H_j leaves alone).  A row needs nothing of
+// the other rows, so a block takes FR rows through all steps in registers,
+// the next reflector on its way while this one is applied; no barrier between
+// blocks.  (A grid barrier per step, rows in L2: 8 us a step at 256 x 512.)
+constexpr int FT = 64;                        // threads
+template <int EPT, int FR>
+__global__ void __launch_bounds__(FT)
+k_lq_formq(const cplx* __restrict__ W, const double* __restrict__ refl, int q, int k, cplx* Qh) {
+  __shared__ double sh[2][FT / 32][8];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  // rows blockIdx.x, blockIdx.x + gridDim.x, ... (a later row starts earlier)
+  int row[FR];
+  cplx y[FR][EPT];
+#pragma unroll
+  for (int r = 0; r < FR; ++r) {
+    row[r] = (int)blockIdx.x + r * (int)gridDim.x;
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) y[r][i] = cmake(tid + FT * i == row[r] ? 1.0 : 0.0, 0.0);
+  }
+  int top = -1;                               // the largest row of this block
+#pragma unroll
+  for (int r = 0; r < FR; ++r)
+    if (row[r] < k) top = max(top, row[r]);
+  cplx x[EPT];
+  auto fetch = [&](int j) {
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) {
+      const int e = tid + FT * i;
+      x[i] = cmake(0.0, 0.0);
+      if (j >= 0 && e >= j && e < q)
+        x[i] = e == j ? cmake(refl[3 * j], refl[3 * j + 1]) : W[(long long)j * q + e];
+    }
+  };
+  fetch(top);
+  for (int j = top; j >= 0; --j) {
+    const double c = refl[3 * j + 2];
+    double v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = 0.0;
+#pragma unroll
+    for (int i = 0; i < EPT; ++i)
+#pragma unroll
+      for (int r = 0; r < FR; ++r) {
+        v[2 * r] = fma(y[r][i].x, x[i].x, fma(y[r][i].y, x[i].y, v[2 * r]));
+        v[2 * r + 1] = fma(y[r][i].y, x[i].x, fma(-y[r][i].x, x[i].y, v[2 * r + 1]));
+      }
+    const double sum = warp_sum8(v);
+    if ((lane & 3) == 0) sh[j & 1][w][lane >> 2] = sum;
+    cplx u[EPT];
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) u[i] = x[i];
+    fetch(j - 1);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < FR; ++r) {
+      double dr = sh[j & 1][0][2 * r], di = sh[j & 1][0][2 * r + 1];
+#pragma unroll
+      for (int b = 1; b < FT / 32; ++b) {
+        dr += sh[j & 1][b][2 * r];
+        di += sh[j & 1][b][2 * r + 1];
+      }
+      // a row above j is a unit vector left of u_j's support: d = 0
+      const double fr = c * dr, fi = c * di;
+#pragma unroll
+      for (int i = 0; i < EPT; ++i) {
+        y[r][i].x -= fr * u[i].x - fi * u[i].y;
+        y[r][i].y -= fr * u[i].y + fi * u[i].x;
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < FR; ++r)
+    if (row[r] < k)
+#pragma unroll
+      for (int i = 0; i < EPT; ++i) {
+        const int e = tid + FT * i;
+        if (e < q) Qh[(long long)row[r] * q + e] = y[r][i];
+      }
+}
+
+// The same for rows of any length, one block per row, the row in Qh.
 __global__ void __launch_bounds__(JT)
-k_lq_formq(const cplx* W, const double* refl, int q, int k, cplx* Qh, unsigned int* st) {
+k_lq_formq_long(const cplx* W, const double* refl, int q, int k, cplx* Qh) {
   __shared__ double sh[2][JT / 32];
-  const unsigned int nb = gridDim.x;
-  for (int j = k - 1; j >= 0; --j) {
+  const int i = blockIdx.x;
+  cplx* y = Qh + (long long)i * q;
+  for (int e = threadIdx.x; e < q; e += JT) y[e] = cmake(e == i ? 1.0 : 0.0, 0.0);
+  for (int j = i; j >= 0; --j) {
     const double c = refl[3 * j + 2];
     const cplx u0 = cmake(refl[3 * j], refl[3 * j + 1]);
     const cplx* x = W + (long long)j * q;
-    if (c != 0.0) {
-      for (int i = j + (int)blockIdx.x; i < k; i += (int)nb) {
-        cplx* y = Qh + (long long)i * q;
-        double dr = 0.0, di = 0.0;     // y u^H
-        for (int e = j + threadIdx.x; e < q; e += JT) {
-          const cplx u = e == j ? u0 : x[e];
-          const cplx v = y[e];
-          dr = fma(v.x, u.x, fma(v.y, u.y, dr));
-          di = fma(v.y, u.x, fma(-v.x, u.y, di));
-        }
-        block_sum2(dr, di, sh);
-        const double fr = c * dr, fi = c * di;
-        for (int e = j + threadIdx.x; e < q; e += JT) {
-          const cplx u = e == j ? u0 : x[e];
-          cplx v = y[e];
-          v.x -= fr * u.x - fi * u.y;
-          v.y -= fr * u.y + fi * u.x;
-          y[e] = v;
-        }
-      }
+    if (c == 0.0) continue;
+    double dr = 0.0, di = 0.0;     // y u^H; a thread reads what it wrote itself
+    for (int e = threadIdx.x; e < q; e += JT) {
+      if (e < j) continue;
+      const cplx u = e == j ? u0 : x[e];
+      const cplx v = y[e];
+      dr = fma(v.x, u.x, fma(v.y, u.y, dr));
+      di = fma(v.y, u.x, fma(-v.x, u.y, di));
     }
-    if (!grid_barrier(st, nb)) return;
+    block_sum2(dr, di, sh);
+    const double fr = c * dr, fi = c * di;
+    for (int e = threadIdx.x; e < q; e += JT) {
+      if (e < j) continue;
+      const cplx u = e == j ? u0 : x[e];
+      cplx v = y[e];
+      v.x -= fr * u.x - fi * u.y;
+      v.y -= fr * u.y + fi * u.x;
+      y[e] = v;
+    }
   }
 }
 
@@ -882,49 +1180,75 @@ __global__ void k_sort_rank(const double* sigma, int p, int* perm, double* sorte
     }
     return;
   }
+  // positions by counting, from a copy in shared memory where it fits
+  __shared__ double ss[4096];
+  const bool staged = p <= 4096;
+  if (staged)
+    for (int i = threadIdx.x; i < p; i += blockDim.x) ss[i] = sigma[i];
+  __syncthreads();
   for (int i = threadIdx.x; i < p; i += blockDim.x) {
     const double si = sigma[i];
     int pos = 0;
+#pragma unroll 4
     for (int j = 0; j < p; ++j) {
-      const double sj = sigma[j];
+      const double sj = staged ? ss[j] : sigma[j];
       pos += (sj > si) || (sj == si && j < i);
     }
     perm[pos] = i;
     sorted[pos] = si;
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
-  // tail[r] = sum_{k >= r} sigma_k^2, accumulated from the smallest value up
+  // tail[r] = sum_{k >= r} sigma_k^2, accumulated from the smallest value up, 32
+  // values at a time: warp 0 scans them backwards (lane 0 the smallest), which
+  // is the order of the oracle's sum up to the tree within the 32
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x;
+  auto weight = [&](int k) { return k >= 0 ? sorted[k] * sorted[k] : 0.0; };
+  auto scan = [&](double v) {
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double t = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += t;
+    }
+    return v;
+  };
   double total = 0.0;
-  for (int k = p - 1; k >= 0; --k) total += sorted[k] * sorted[k];
-  int r = p;
+  for (int k0 = p - 1; k0 >= 0; k0 -= 32)
+    total += __shfl_sync(0xffffffffu, scan(weight(k0 - lane)), 31);
   if (total == 0.0) {
-    *rank_out = 1;
-    *disc_out = 0.0;
+    if (lane == 0) {
+      *rank_out = 1;
+      *disc_out = 0.0;
+    }
     return;
   }
   const double tol = (cutoff > floor_w ? cutoff : floor_w) * total;
-  // find the smallest r >= 1 with tail[r] <= tol: walk up from the end
-  {
-    double tail = 0.0;     // tail[p] = 0
-    int best = p;
-    for (int cand = p; cand >= 1; --cand) {
-      // tail currently = tail[cand]
-      if (tail <= tol) best = cand; else break;
-      tail += sorted[cand - 1] * sorted[cand - 1];
-    }
-    r = best;
+  // the smallest r >= 1 with tail[r] <= tol
+  int r = p;
+  double base = 0.0;                     // tail of the values already walked past
+  for (int k0 = p - 1; k0 >= 0; k0 -= 32) {
+    const double t = base + scan(weight(k0 - lane));      // tail[k0 - lane]
+    const unsigned int fits = __ballot_sync(0xffffffffu, k0 - lane >= 1 && t <= tol);
+    // tails grow with the lane: the lanes that fit come first
+    const int n = fits == 0xffffffffu ? 32 : __ffs((int)~fits) - 1;
+    r -= n;
+    if (n < 32) break;
+    base = __shfl_sync(0xffffffffu, t, 31);
   }
   if (r > chi_max) r = chi_max;
-  if (r < p && sorted[r] >= sorted[r - 1] * (1.0 - tie_rel)) {
+  if (lane == 0 && r < p && sorted[r] >= sorted[r - 1] * (1.0 - tie_rel)) {
     int g = r - 1;
     while (g > 0 && sorted[g] >= sorted[g - 1] * (1.0 - tie_rel)) --g;
     if (g >= 1) r = g;
   }
+  r = __shfl_sync(0xffffffffu, r, 0);
   double tail = 0.0;
-  for (int k = p - 1; k >= r; --k) tail += sorted[k] * sorted[k];
-  *rank_out = r;
-  *disc_out = tail / total;
+  for (int k0 = p - 1; k0 >= r; k0 -= 32)
+    tail += __shfl_sync(0xffffffffu, scan(k0 - lane >= r ? weight(k0 - lane) : 0.0), 31);
+  if (lane == 0) {
+    *rank_out = r;
+    *disc_out = tail / total;
+  }
 }
 
 // Uh[k][i] = D[perm[k]][i] / sorted[k]; a zero row (only for X = 0, rank 1)
@@ -986,7 +1310,7 @@ struct Coresident {
     return b > 0 ? cudaSuccess : cudaErrorInvalidConfiguration;
   }
 };
-Coresident g_lq_blocks, g_jacobi_blocks, g_formq_blocks, g_jgroup_blocks;
+Coresident g_lq_blocks, g_jacobi_blocks, g_jgroup_blocks;
 
 // The grid barrier of the cooperative kernels with `absent` blocks that never
 // arrive: the others wait until the barrier's iteration limit, set the error
@@ -1006,11 +1330,49 @@ cudaError_t barrier_selftest(unsigned int* dev_state, int blocks, int absent, cu
   return cudaLaunchCooperativeKernel((void*)k_barrier_selftest, dim3(blocks), dim3(32), args, 0, st);
 }
 
-cudaError_t svd_lq(cplx* W, int p, int q, cplx* beta, double* refl, unsigned int* dev_state,
-                   cudaStream_t st) {
+namespace {
+
+constexpr size_t kLqSmemMax = 200 * 1024;
+
+// k_lq_resident with EPT elements per thread: tried = false if its rows do not
+// fit the SMs' shared memory
+template <int EPT>
+cudaError_t launch_lq_resident(cplx* W, int p, int q, cplx* beta, double* refl, cplx* pub,
+                               unsigned int* st, int sms, cudaStream_t s, bool* tried) {
+  const int nb = p < sms ? p : sms;
+  const size_t smem = (size_t)((p + nb - 1) / nb) * EPT * LT * sizeof(cplx);
+  *tried = smem <= kLqSmemMax;
+  if (!*tried) return cudaSuccess;
+  cudaError_t err = cudaFuncSetAttribute(k_lq_resident<EPT>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLqSmemMax);
+  if (err != cudaSuccess) return err;
+  const int k = p < q ? p : q;
+  err = cudaMemsetAsync(pub, 0xFF, (size_t)k * q * sizeof(cplx), s);
+  if (err != cudaSuccess) return err;
+  void* args[] = {&W, &p, &q, &beta, &refl, &pub, &st};
+  count_launches(1);
+  return cudaLaunchCooperativeKernel((void*)k_lq_resident<EPT>, dim3(nb), dim3(LT), args, smem, s);
+}
+
+}  // namespace
+
+cudaError_t svd_lq(cplx* W, int p, int q, cplx* beta, double* refl, cplx* pub,
+                   unsigned int* dev_state, cudaStream_t st) {
   cudaError_t err = cudaMemsetAsync(dev_state, 0, 8 * sizeof(unsigned int), st);
   if (err != cudaSuccess) return err;
   if (p < 1 || q < 1) return cudaSuccess;
+  int sms = 0, dev = 0;
+  err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (err != cudaSuccess) return err;
+  bool tried = false;
+  if (q <= 2 * LT) err = launch_lq_resident<2>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
+  else if (q <= 4 * LT) err = launch_lq_resident<4>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
+  else if (q <= 8 * LT) err = launch_lq_resident<8>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
+  else if (q <= 16 * LT) err = launch_lq_resident<16>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
+  if (tried || err != cudaSuccess) return err;
+  // larger blocks: the rows in L2, one grid barrier per step
   int max_blocks = 0;
   err = g_lq_blocks.get((const void*)k_lq_persistent, JT, &max_blocks);
   if (err != cudaSuccess) return err;
@@ -1045,21 +1407,16 @@ cudaError_t lq_inv_fnorm2(const cplx* W, const cplx* beta, int q, int k, double*
   return cudaGetLastError();
 }
 
-cudaError_t lq_formq(const cplx* W, const double* refl, int q, int k, cplx* Qh,
-                     unsigned int* dev_state, cudaStream_t st) {
-  cudaError_t err = cudaMemsetAsync(dev_state, 0, 8 * sizeof(unsigned int), st);
-  if (err != cudaSuccess) return err;
+cudaError_t lq_formq(const cplx* W, const double* refl, int q, int k, cplx* Qh, cudaStream_t st) {
   if (k < 1) return cudaSuccess;
   count_launches(1);
-  k_eye_rows<<<grid_for((long long)k * q), 256, 0, st>>>(Qh, k, q);
-  int max_blocks = 0;
-  err = g_formq_blocks.get((const void*)k_lq_formq, JT, &max_blocks);
-  if (err != cudaSuccess) return err;
-  int nblk = k;
-  if (nblk > max_blocks) nblk = max_blocks;
-  void* args[] = {&W, &refl, &q, &k, &Qh, &dev_state};
-  count_launches(1);
-  return cudaLaunchCooperativeKernel((void*)k_lq_formq, dim3(nblk), dim3(JT), args, 0, st);
+  const int half = (k + 1) / 2;
+  if (q <= 2 * FT) k_lq_formq<2, 2><<<half, FT, 0, st>>>(W, refl, q, k, Qh);
+  else if (q <= 4 * FT) k_lq_formq<4, 2><<<half, FT, 0, st>>>(W, refl, q, k, Qh);
+  else if (q <= 8 * FT) k_lq_formq<8, 2><<<half, FT, 0, st>>>(W, refl, q, k, Qh);
+  else if (q <= 16 * FT) k_lq_formq<16, 1><<<k, FT, 0, st>>>(W, refl, q, k, Qh);
+  else k_lq_formq_long<<<k, JT, 0, st>>>(W, refl, q, k, Qh);
+  return cudaGetLastError();
 }
 
 cudaError_t svd_lq_r(const cplx* W, const cplx* beta, int p, int q, cplx* R, cudaStream_t st) {

@@ -100,3 +100,32 @@ def test_split_of_zero_and_non_finite_blocks(api, ctx):
     # the context still works
     r, _, sig, _, _ = _split(api, ctx, np.nan_to_num(X), 40, 0.0, True, True)
     assert r == 40
+
+
+@pytest.mark.parametrize("m,n", [(20, 127), (20, 129), (257, 20), (30, 513), (1025, 24), (3, 2050),
+                                 (200, 1030)])
+def test_split_of_long_rows(api, ctx, m, n):
+    # the Householder LQ's variants by row length, and its general form beyond them
+    X = _matrix(np.random.default_rng(m + n), m, n, "decay")
+    S = np.linalg.svd(X, compute_uv=False)
+    p, tol = min(m, n), 16 * max(m, n) * EPS
+    for right in (True, False):
+        r, disc, sig, L, R = _split(api, ctx, X, p, 0.0, right, True)
+        assert r == p
+        assert np.abs(sig - S).max() <= tol * S[0]
+        assert np.linalg.norm(L @ R - X) <= tol * np.linalg.norm(X) + 1e-12 * S[0]
+
+
+@pytest.mark.parametrize("chi,N", [(6, 8), (40, 14), (100, 16), (200, 18), (300, 20), (600, 22)])
+def test_gauge_move_is_isometric_and_keeps_the_state(api, ctx, chi, N):
+    # rows of 12 to 1200: every variant of the reflectors' accumulation
+    from paper_2606_02930_gb300 import inputs
+    A = inputs.random_isometric_mps(N, 2, chi, chi, kappa=chi / 4)
+    psi = api.mps_create(ctx, A, chi)
+    ref = api.mps_create(ctx, A, chi)
+    api.mps_sample(ctx, psi, np.full(N, 0.5))
+    nn = api.overlap(ctx, ref, ref).real
+    assert abs(api.overlap(ctx, ref, psi) - nn) <= 64 * 2 * chi * EPS * nn
+    for T in psi.tensors()[1:]:
+        M = T.reshape(T.shape[0], -1)
+        assert np.abs(M @ M.conj().T - np.eye(M.shape[0])).max() <= 16 * M.shape[1] * EPS
