@@ -62,6 +62,7 @@ struct Pre32 {
   float2* V;                                  // kp rows of vl, the accumulated rotation
   int k, kp, pl, vl, nb;                      // rows, padded rows, row strides, blocks
   int pc, vc, chunk;                          // columns of R and V per CTA, columns staged at once
+  unsigned int* ver;                          // (block, CTA of a cluster): steps done
 };
 
 // Barrier over the clusters' first CTAs: arrivals are counted up without a reset,
@@ -102,6 +103,12 @@ __device__ __forceinline__ void copy16(float2* dst, const float4* src) {
                : "memory");
 }
 
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -111,32 +118,169 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // Rotation x' = c x - s y, y' = conj(s) x + c y of two rows with squared norms
 // al, be and inner product g = x y^H that makes them orthogonal; returns what it
 // moves from al to be.  Written in the overlap h = g / (|x| |y|) and the ratio of
-// the norms, which stay in range for rows of any weight, and in approximate
-// reciprocals and square roots (the chain of them is what a round waits for);
-// c is refined by a Newton step so that |c|^2 + |s|^2 = 1 to rounding.
+// the norms, which stay in range for rows of any weight: with zeta = (be - al) /
+// (2 |g|) and r = 1 / sqrt(1 + zeta^2), cos 2a = |zeta| r and sin 2a = r, so
+// c^2 = (1 + |zeta| r) / 2 and |s| = r / (2 c).  Every round waits for this chain:
+// four dependent approximate inverse square roots and no branch; the last two are
+// refined by a Newton step so that c^2 + |s|^2 = 1 to rounding.
 __device__ __forceinline__ float rotation(float al, float be, float2 g, float& c, float& sx,
                                           float& sy, float& off) {
-  c = 1.f;
-  sx = sy = 0.f;
-  if (!(al > kTiny32 && be > kTiny32)) return 0.f;
-  const float ra = rsqrtf(al), rb = rsqrtf(be);
-  const float hx = g.x * ra * rb, hy = g.y * ra * rb;
+  const bool rows = al > kTiny32 && be > kTiny32;
+  const float ra = rsqrt_approx(rows ? al : 1.f), rb = rsqrt_approx(rows ? be : 1.f);
+  const float rab = ra * rb, hx = g.x * rab, hy = g.y * rab;
   const float h2 = fmaf(hx, hx, hy * hy);
-  if (!(h2 > kRot32 * kRot32)) return 0.f;
-  const float ih = rsqrtf(h2), h = h2 * ih;
-  off = fmaxf(off, h);
-  // zeta = (be - al) / (2 |g|), tangent t = 1 / (|zeta| + sqrt(1 + zeta^2))
-  const float q = be * rb * ra, qi = al * ra * rb;
-  const float z = 0.5f * (q - qi) * ih, az = fabsf(z);
-  const float w = fmaf(z, z, 1.f);
-  const float t = rcp_approx(az < 1e9f ? az + w * rsqrtf(w) : az + az);
-  const float d = fmaf(t, t, 1.f);
-  c = rsqrtf(d);
-  c = c * fmaf(-0.5f * d * c, c, 1.5f);
-  const float sg = copysignf(c * t * ih, z);
-  sx = sg * hx;
-  sy = sg * hy;
-  return copysignf(t * h * (al * ra) * (be * rb), z);
+  const bool on = rows && h2 > kRot32 * kRot32;
+  const float ih = rsqrt_approx(on ? h2 : 1.f);
+  const float df = be - al;
+  const float z = 0.5f * fabsf(df) * rab * ih;
+  // r = 1 / z where 1 + z^2 is z^2 (and may be infinite): s has to stay exact, it
+  // multiplies a row that can be 1e17 times as long as the other
+  const bool far = z > 1e9f;
+  const float w = fmaf(z, z, 1.f), rf = rcp_approx(z);
+  float r = rsqrt_approx(w);
+  r = far ? rf : r * fmaf(-0.5f * w * r, r, 1.5f);
+  const float c2 = far ? 1.f : fmaf(0.5f * z, r, 0.5f);
+  float q = rsqrt_approx(c2);
+  q = q * fmaf(-0.5f * c2 * q, q, 1.5f);      // 1 / c
+  const float sn = on ? copysignf(0.5f * r * q * ih, df) : 0.f;
+  c = on ? c2 * q : 1.f;
+  sx = sn * hx;
+  sy = sn * hy;
+  off = fmaxf(off, on ? h2 * ih : 0.f);
+  // t |g| = (|s| / c) |h| |x| |y|
+  return sn * q * h2 * (al * ra) * (be * rb);
+}
+
+// Columns of one rank of a block have been through `step` steps: each CTA needs
+// nothing but its own columns of the two blocks, so it waits for the CTAs that
+// wrote these instead of for all.  Bounded; after a failed wait anywhere the
+// sweep is run out without waiting (its result is discarded).
+__device__ __forceinline__ void wait_block(const unsigned int* ver, unsigned int step,
+                                           unsigned int* st) {
+  for (unsigned int spins = 0;; ++spins) {
+    unsigned int seen;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(ver) : "memory");
+    if ((int)(seen - step) >= 0) return;
+    if ((spins & 63u) == 63u && *((volatile unsigned int*)(st + C_ERR)) != 0u) return;
+    if (spins > (1u << 24)) {
+      atomicExch(st + C_ERR, 1u);
+      return;
+    }
+  }
+}
+
+__device__ __forceinline__ void publish_block(unsigned int* ver, unsigned int step) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(ver), "r"(step) : "memory");
+}
+
+__device__ __forceinline__ float2 conj(const float2& a) { return make_float2(a.x, -a.y); }
+__device__ __forceinline__ float2 neg(const float2& a) { return make_float2(-a.x, -a.y); }
+
+// c x + f y in this order of operations wherever it stands.
+__device__ __forceinline__ float2 turn(float c, const float2& x, const float2& f, const float2& y) {
+  return make_float2(fmaf(c, x.x, fmaf(f.x, y.x, -__fmul_rn(f.y, y.y))),
+                     fmaf(c, x.y, fmaf(f.x, y.y, __fmul_rn(f.y, y.x))));
+}
+
+// Where the entries of round r + 1's pair t stand before round r has turned them:
+// pair (m, n = m ^ (r + 1)), the partners m_ = m ^ r, n_ = n ^ r of round r, the
+// pairs pm, pn of round r that m and n are in, and 1 or -1 as they are the second
+// or the first there.  m and n are exchanged (swap) where that puts the lower pair
+// first, as in the update's blocks.
+struct Ahead {
+  int mn, mn_, m_n, m_n_, mm, nn, pm, pn;
+  float sm, sn;
+  bool swap;
+  __device__ __forceinline__ Ahead(int r, int t) {
+    const int r2 = min(r + 1, PM - 1);
+    const int hb = 31 - __clz(r), low = (1 << hb) - 1, low2 = (1 << (31 - __clz(r2))) - 1;
+    int m = ((t & ~low2) << 1) | (t & low2), n = m ^ r2;
+    auto index = [&](int x) {
+      const int f = (x >> hb) & 1 ? x ^ r : x;
+      return ((f >> 1) & ~low) | (f & low);
+    };
+    pm = index(m);
+    pn = index(n);
+    swap = pm > pn;
+    if (swap) {
+      int x = m;
+      m = n;
+      n = x;
+      x = pm;
+      pm = pn;
+      pn = x;
+    }
+    mn = m * GLD + n;
+    mn_ = m * GLD + (n ^ r);
+    m_n = (m ^ r) * GLD + n;
+    m_n_ = (m ^ r) * GLD + (n ^ r);
+    mm = m * (GLD + 1);
+    nn = n * (GLD + 1);
+    sm = (m >> hb) & 1 ? 1.f : -1.f;
+    sn = (n >> hb) & 1 ? 1.f : -1.f;
+  }
+};
+
+// Rows m, n of N columns of Q, STEP apart, turned by the rotation A = (c, s).
+template <int N, int STEP>
+__device__ __forceinline__ void turn_q(float2* q, int m, int n, const float4& A) {
+  const float2 sn = make_float2(A.y, A.z);
+  float2 x[N], y[N];
+#pragma unroll
+  for (int h = 0; h < N; ++h) {
+    x[h] = q[h * STEP * QLD + m];
+    y[h] = q[h * STEP * QLD + n];
+  }
+#pragma unroll
+  for (int h = 0; h < N; ++h) {
+    q[h * STEP * QLD + m] = turn(A.x, x[h], neg(sn), y[h]);
+    q[h * STEP * QLD + n] = turn(A.x, y[h], conj(sn), x[h]);
+  }
+}
+
+// Rows r0..r0+7 of Q S for NC columns per lane, written to their sorted places.
+template <int NC>
+__device__ __forceinline__ void apply_rows(const Pre32& a, const float2* S, const float2* QT,
+                                           const int* pos, int ld, int cb, int n, int r0, int u,
+                                           int v, int rank, int c0) {
+  const int lane = threadIdx.x & 31, half = threadIdx.x >> 7;
+  const int c = cb + 32 * half + lane;
+  const float2* sp[NC];
+#pragma unroll
+  for (int j = 0; j < NC; ++j) sp[j] = S + (c + 64 * j < n ? c + 64 * j : 0);
+  float2 o[8][NC];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < NC; ++j) o[i][j] = make_float2(0.f, 0.f);
+#pragma unroll 4
+  for (int m = 0; m < PM; ++m) {
+    float2 s[NC];
+#pragma unroll
+    for (int j = 0; j < NC; ++j) s[j] = sp[j][m * ld];
+    const float4* qp = reinterpret_cast<const float4*>(QT + m * QLD + r0);
+#pragma unroll
+    for (int i2 = 0; i2 < 4; ++i2) {
+      const float4 q = qp[i2];
+#pragma unroll
+      for (int j = 0; j < NC; ++j) {
+        float2& o0 = o[2 * i2][j];
+        float2& o1 = o[2 * i2 + 1][j];
+        o0.x = fmaf(q.x, s[j].x, fmaf(-q.y, s[j].y, o0.x));
+        o0.y = fmaf(q.x, s[j].y, fmaf(q.y, s[j].x, o0.y));
+        o1.x = fmaf(q.z, s[j].x, fmaf(-q.w, s[j].y, o1.x));
+        o1.y = fmaf(q.z, s[j].y, fmaf(q.w, s[j].x, o1.y));
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int at = pos[r0 + i];
+    const int row = at < PB ? u * PB + at : v * PB + at - PB;
+#pragma unroll
+    for (int j = 0; j < NC; ++j)
+      if (c + 64 * j < n) *reinterpret_cast<float2*>(col_ptr(a, row, rank, c0 + c + 64 * j)) = o[i][j];
+  }
 }
 
 // One cluster per block pair, the columns of the pair's rows dealt to its
@@ -145,30 +289,33 @@ __device__ __forceinline__ float rotation(float al, float be, float2 g, float& c
 // fixed order, every CTA diagonalises the sum the same way and applies the
 // result to its own columns.
 // Bound: latency and shared memory.  Clocks per step at k = 512 (16 pairs, 6 CTAs
-// each, 31 steps a sweep): copy in 2.2k, Gram 5.8k, sum 3.8k, the 16 or 31
-// dependent rounds 18k (900 each: the chain of approximate square roots, then
-// the two-sided update), rows 12k, grid barrier 6.9k; 23.7 us in all.  16-row
-// blocks: 8-row ones need twice the steps and barriers for the same number of
-// rounds, 32-row ones leave half the SMs without a pair.  Whole 512 x 512 split
-// (chi_max 256, cutoff 1e-10): 69.9 ms with the FP64 Jacobi alone, 13.9 ms with
-// the preconditioner (no FP64 sweep is left); 1024 x 1024: 325 ms and 54.6 ms.
-__global__ void __launch_bounds__(PT)
+// each, 31 steps a sweep): wait for the blocks 1.7k, copy in 1.7k, Gram 4.3k, sum
+// 3.3k, the 16 or 31 dependent rounds 13.8k (620 each: the chain of approximate
+// square roots on warp 4), rows 12k; 19 us in all.  With a barrier over the grid
+// after every step, the rotations formed before the update and 2 x 2 tiles in the
+// Gram matrix: 23.7 us.  16-row blocks: 8-row ones need twice the steps for the
+// same number of rounds, 32-row ones leave half the SMs without a pair.  Whole
+// 512 x 512 split (chi_max 256, cutoff 1e-10): 69 ms with the FP64 Jacobi alone,
+// 9.0 ms with the preconditioner (no FP64 sweep is left); 1024 x 1024: 325 and 35.
+__global__ void __launch_bounds__(PT, 1)
 k_jacobi32(Pre32 a, unsigned int* st) {
   cg::cluster_group cl = cg::this_cluster();
   const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int ncl = gridDim.x / C, cid = blockIdx.x / C;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   extern __shared__ float4 dyn[];
-  float2* part = reinterpret_cast<float2*>(dyn);            // PM x GLD
-  float2* G = part + PM * GLD;                              // PM x GLD
+  float2* parts = reinterpret_cast<float2*>(dyn);           // PM x GLD, by parity of the pair
+  float2* G = parts + 2 * PM * GLD;                         // PM x GLD
   float2* G2 = G + PM * GLD;                                // PM x GLD
   float2* QT = G2 + PM * GLD;                               // PM x QLD: QT[c][r] = Q[r][c]
   float2* S = QT + PM * QLD;                                // PM x ld
   __shared__ int s_pos[PM];
   __shared__ int s_off, s_ok;
+  __shared__ float4 s_rot[2][PB];             // rotations (c, s, t |g|) of a round, by its parity
   const int lc = a.pc + a.vc, ld = a.chunk + 2;
   const bool resident = lc <= a.chunk;
-  const int ty = tid >> 4, tx = tid & 15;
+  const int tx = tid & 15;
+  const int gk = tid >> 6, gi = (tid >> 3) & 7, gj = tid & 7;      // of the Gram matrix
   unsigned int passed = 0;                    // barrier arrivals so far
   // the two row pairs pa < pb whose block of G this thread turns (tid < 120):
   // rows x and 15 - x of the 16 x 16 triangle make one row of 15 blocks
@@ -187,47 +334,73 @@ k_jacobi32(Pre32 a, unsigned int* st) {
     asm volatile("cp.async.wait_all;" ::: "memory");
   };
 
+  int pairs_done = 0;
   for (int sw = 0; sw < kSweeps32; ++sw) {
-    bool ok = true;
     for (int rd = 0; rd < a.nb - 1; ++rd) {
-      for (int k = cid; k < a.nb / 2; k += ncl) {
+      const unsigned int step = (unsigned int)(sw * (a.nb - 1) + rd);
+      for (int k = cid; k < a.nb / 2; k += ncl, ++pairs_done) {
         int u = seat(k, rd, a.nb), v = seat(a.nb - 1 - k, rd, a.nb);
         if (u > v) { const int t = u; u = v; v = t; }
-        // ---- share of the Gram matrix: thread (ty, tx) rows ty, ty+16 by tx, tx+16
-        float2 acc[2][2];
+        // this CTA's columns of the two blocks, as the last step left them
+        if (tid == 0) {
+          wait_block(a.ver + u * 8 + rank, step, st);
+          wait_block(a.ver + v * 8 + rank, step, st);
+        }
+        __syncthreads();
+        float2* const part = parts + (pairs_done & 1) * PM * GLD;
+        // ---- share of the Gram matrix: four groups of 64 threads take every
+        // fourth pair of columns, thread (gi, gj) of a group the rows gi + 8 x by
+        // gj + 8 y, x <= y (the others are mirror images)
+        float2 acc[10];
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
-#pragma unroll
-          for (int j = 0; j < 2; ++j) acc[i][j] = make_float2(0.f, 0.f);
+        for (int i = 0; i < 10; ++i) acc[i] = make_float2(0.f, 0.f);
         for (int c0 = 0; c0 < (resident ? 1 : a.pc); c0 += a.chunk) {
           const int n = resident ? lc : min(a.chunk, a.pc - c0);
           const int ng = resident ? a.pc : n;
           stage(u, v, c0, n);
           __syncthreads();
-          for (int c = 0; c < ng; c += 2) {
-            float4 x[2], y[2];
+          for (int c = 2 * gk; c < ng; c += 8) {
+            float4 x[4], y[4];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-              x[i] = *reinterpret_cast<const float4*>(S + (ty + PB * i) * ld + c);
-              y[i] = *reinterpret_cast<const float4*>(S + (tx + PB * i) * ld + c);
+            for (int i = 0; i < 4; ++i) {
+              x[i] = *reinterpret_cast<const float4*>(S + (gi + 8 * i) * ld + c);
+              y[i] = *reinterpret_cast<const float4*>(S + (gj + 8 * i) * ld + c);
             }
+            int e = 0;
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-              for (int j = i; j < 2; ++j) {
-                // x conj(y) (rows ty + 16 by tx mirror others' ty by tx + 16)
-                acc[i][j].x = fmaf(x[i].x, y[j].x, fmaf(x[i].y, y[j].y, acc[i][j].x));
-                acc[i][j].y = fmaf(x[i].y, y[j].x, fmaf(-x[i].x, y[j].y, acc[i][j].y));
-                acc[i][j].x = fmaf(x[i].z, y[j].z, fmaf(x[i].w, y[j].w, acc[i][j].x));
-                acc[i][j].y = fmaf(x[i].w, y[j].z, fmaf(-x[i].z, y[j].w, acc[i][j].y));
+              for (int j = i; j < 4; ++j, ++e) {
+                // x conj(y)
+                acc[e].x = fmaf(x[i].x, y[j].x, fmaf(x[i].y, y[j].y, acc[e].x));
+                acc[e].y = fmaf(x[i].y, y[j].x, fmaf(-x[i].x, y[j].y, acc[e].y));
+                acc[e].x = fmaf(x[i].z, y[j].z, fmaf(x[i].w, y[j].w, acc[e].x));
+                acc[e].y = fmaf(x[i].w, y[j].z, fmaf(-x[i].z, y[j].w, acc[e].y));
               }
           }
           if (!resident) __syncthreads();
         }
+        // groups 1-3 hand theirs to group 0 (G, G2 and QT are free here)
+        float2* const mine = gk == 0 ? part : gk == 1 ? G : gk == 2 ? G2 : QT;
+        if (gk > 0) {
+          int e = 0;
 #pragma unroll
-        for (int i = 0; i < 2; ++i)
+          for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = i; j < 2; ++j) part[(ty + PB * i) * GLD + tx + PB * j] = acc[i][j];
+            for (int j = i; j < 4; ++j, ++e) mine[(gi + 8 * i) * GLD + gj + 8 * j] = acc[e];
+        }
+        __syncthreads();
+        if (gk == 0) {
+          int e = 0;
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = i; j < 4; ++j, ++e) {
+              const int at = (gi + 8 * i) * GLD + gj + 8 * j;
+              const float2 p = G[at], q = G2[at], r = QT[at];
+              part[at] = make_float2((acc[e].x + p.x) + (q.x + r.x), (acc[e].y + p.y) + (q.y + r.y));
+            }
+        }
         cl.sync();
         // ---- sum of the shares (upper triangle, mirrored); Q = I
         for (int e = tid; e < PM * (PM + 1) / 2; e += PT) {
@@ -261,72 +434,88 @@ k_jacobi32(Pre32 a, unsigned int* st) {
         // fourth step, only those across the two blocks (16 rounds instead of
         // 31) in the others: as many sweeps as with all pairs every time.
         // Round r pairs row i with row i ^ r; pair t is the t-th i whose highest
-        // bit of r is clear.  Lane t of every warp forms the rotation of pair
-        // t.  Warps 0-3 turn the 120 blocks of two different pairs from one copy
-        // of G to the other (upper block, mirrored), warps 4-7 the rows of Q
-        // and the pairs' own blocks, so one barrier a round is enough.
+        // bit of r is clear.  Warps 0-3 turn the 120 blocks of two different pairs
+        // from one copy of G to the other (upper block, mirrored), warps 5-7 the
+        // pairs' own blocks and half of Q (warps 0-3 the other half).  Warp 4
+        // meanwhile turns just the entries that the next round's pairs need and
+        // forms their rotations, so that the chain of square roots runs beside the
+        // update, not before it: 620 clocks a round, 850 one after the other.
         float off = 0.f;
         float2 *Ga = G, *Gb = G2;
-        for (int r = (rd & 3) == 0 ? 1 : PB; r < PM; ++r) {
+        const int rfirst = (rd & 3) == 0 ? 1 : PB;
+        if (warp == 4) {
+          const int hb = 31 - __clz(rfirst), low = (1 << hb) - 1;
+          const int m = ((tx & ~low) << 1) | (tx & low), n = m ^ rfirst;
+          float4 q;
+          q.w = rotation(Ga[m * GLD + m].x, Ga[n * GLD + n].x, Ga[m * GLD + n], q.x, q.y, q.z, off);
+          if (lane < PB) s_rot[rfirst & 1][tx] = q;
+        }
+        Ahead ahead(rfirst, tx);
+        __syncthreads();
+        for (int r = rfirst; r < PM; ++r) {
           const int hb = 31 - __clz(r), low = (1 << hb) - 1;
           auto first = [&](int t) { return ((t & ~low) << 1) | (t & low); };
-          const int m = first(tx), n = m ^ r;
-          const float al = Ga[m * GLD + m].x, be = Ga[n * GLD + n].x;
-          const float2 g = Ga[m * GLD + n];
+          const float4* const rot = s_rot[r & 1];
           if (warp < 4) {
-            const int i = first(pa), j = i ^ r, k2 = first(pb), l2 = k2 ^ r;
-            const float2 b00 = Ga[i * GLD + k2], b01 = Ga[i * GLD + l2];
-            const float2 b10 = Ga[j * GLD + k2], b11 = Ga[j * GLD + l2];
-            float c, sx, sy;
-            rotation(al, be, g, c, sx, sy, off);
-            const float ca = __shfl_sync(0xffffffffu, c, pa), cb = __shfl_sync(0xffffffffu, c, pb);
-            const float xa = __shfl_sync(0xffffffffu, sx, pa), xb = __shfl_sync(0xffffffffu, sx, pb);
-            const float ya = __shfl_sync(0xffffffffu, sy, pa), yb = __shfl_sync(0xffffffffu, sy, pb);
+            const int mq = first(tx);
+            turn_q<2, 8>(QT + (16 + (tid >> 4)) * QLD, mq, mq ^ r, rot[tx]);
             if (tid < 120) {
+              const int i = first(pa), j = i ^ r, k2 = first(pb), l2 = k2 ^ r;
+              const float4 A = rot[pa], B = rot[pb];
+              const float2 b00 = Ga[i * GLD + k2], b01 = Ga[i * GLD + l2];
+              const float2 b10 = Ga[j * GLD + k2], b11 = Ga[j * GLD + l2];
+              const float2 sa = make_float2(A.y, A.z), sb = make_float2(B.y, B.z);
               // rows: x' = c x - s y, y' = conj(s) x + c y
-              float2 p00, p01, p10, p11;
-              p00.x = ca * b00.x - (xa * b10.x - ya * b10.y);
-              p00.y = ca * b00.y - (xa * b10.y + ya * b10.x);
-              p01.x = ca * b01.x - (xa * b11.x - ya * b11.y);
-              p01.y = ca * b01.y - (xa * b11.y + ya * b11.x);
-              p10.x = (xa * b00.x + ya * b00.y) + ca * b10.x;
-              p10.y = (xa * b00.y - ya * b00.x) + ca * b10.y;
-              p11.x = (xa * b01.x + ya * b01.y) + ca * b11.x;
-              p11.y = (xa * b01.y - ya * b01.x) + ca * b11.y;
+              const float2 p00 = turn(A.x, b00, neg(sa), b10), p01 = turn(A.x, b01, neg(sa), b11);
+              const float2 p10 = turn(A.x, b10, conj(sa), b00), p11 = turn(A.x, b11, conj(sa), b01);
               // columns: x' = c x - conj(s) y, y' = s x + c y
-              auto put = [&](int row, int col, float x, float y) {
-                Gb[row * GLD + col] = make_float2(x, y);
-                Gb[col * GLD + row] = make_float2(x, -y);
+              auto put = [&](int row, int col, const float2& v) {
+                Gb[row * GLD + col] = v;
+                Gb[col * GLD + row] = conj(v);
               };
-              put(i, k2, cb * p00.x - (xb * p01.x + yb * p01.y), cb * p00.y - (xb * p01.y - yb * p01.x));
-              put(i, l2, (xb * p00.x - yb * p00.y) + cb * p01.x, (xb * p00.y + yb * p00.x) + cb * p01.y);
-              put(j, k2, cb * p10.x - (xb * p11.x + yb * p11.y), cb * p10.y - (xb * p11.y - yb * p11.x));
-              put(j, l2, (xb * p10.x - yb * p10.y) + cb * p11.x, (xb * p10.y + yb * p10.x) + cb * p11.y);
+              put(i, k2, turn(B.x, p00, neg(conj(sb)), p01));
+              put(i, l2, turn(B.x, p01, sb, p00));
+              put(j, k2, turn(B.x, p10, neg(conj(sb)), p11));
+              put(j, l2, turn(B.x, p11, sb, p10));
+            }
+          } else if (warp == 4) {
+            if (r + 1 < PM) {
+              // entry (m, n) of the next round's pair: row and column of it are
+              // each turned with their partner m ^ r, n ^ r of this round
+              const Ahead at = ahead;
+              const float4 A = rot[at.pm], B = rot[at.pn];
+              const float2 g0 = Ga[at.mn], g1 = Ga[at.mn_], g2 = Ga[at.m_n], g3 = Ga[at.m_n_];
+              const float am = Ga[at.mm].x, an = Ga[at.nn].x;
+              ahead = Ahead(r + 1, tx);             // in the shadow of the chain below
+              // the same operations as the update's, so that both see one G
+              const float2 fa = make_float2(at.sm * A.y, -A.z), fb = make_float2(at.sn * B.y, B.z);
+              float2 g = turn(B.x, turn(A.x, g0, fa, g2), fb, turn(A.x, g1, fa, g3));
+              float al = fmaf(at.sm, A.w, am), be = fmaf(at.sn, B.w, an);
+              if (at.swap) {
+                const float t = al;
+                al = be;
+                be = t;
+                g.y = -g.y;
+              }
+              float4 q;
+              q.w = rotation(al, be, g, q.x, q.y, q.z, off);
+              if (lane < PB) s_rot[(r + 1) & 1][tx] = q;
             }
           } else {
-            // rows m, n of Q, four columns of it
-            float2* const q = QT + (2 * (warp - 4) + (lane >> 4)) * QLD;
-            float2 x[4], y[4];
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              x[h] = q[8 * h * QLD + m];
-              y[h] = q[8 * h * QLD + n];
-            }
-            float c, sx, sy;
-            const float d = rotation(al, be, g, c, sx, sy, off);
-            if (warp == 4 && lane < PB) {
-              const float2 z = sx != 0.f || sy != 0.f ? make_float2(0.f, 0.f) : g;
-              Gb[m * GLD + m] = make_float2(al - d, 0.f);
-              Gb[n * GLD + n] = make_float2(be + d, 0.f);
-              Gb[m * GLD + n] = z;
-              Gb[n * GLD + m] = make_float2(z.x, -z.y);
-            }
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              q[8 * h * QLD + m] = make_float2(c * x[h].x - (sx * y[h].x - sy * y[h].y),
-                                               c * x[h].y - (sx * y[h].y + sy * y[h].x));
-              q[8 * h * QLD + n] = make_float2((sx * x[h].x + sy * x[h].y) + c * y[h].x,
-                                               (sx * x[h].y - sy * x[h].x) + c * y[h].y);
+            const float4 A = rot[tx];
+            const int m = first(tx), n = m ^ r;
+            if (warp == 5) {
+              if (lane < PB) {
+                const float2 g = Ga[m * GLD + n];
+                const float al = Ga[m * GLD + m].x, be = Ga[n * GLD + n].x;
+                const float2 z = A.y != 0.f || A.z != 0.f ? make_float2(0.f, 0.f) : g;
+                Gb[m * GLD + m] = make_float2(al - A.w, 0.f);
+                Gb[n * GLD + n] = make_float2(be + A.w, 0.f);
+                Gb[m * GLD + n] = z;
+                Gb[n * GLD + m] = make_float2(z.x, -z.y);
+              }
+            } else {
+              turn_q<4, 4>(QT + (2 * (warp - 6) + (lane >> 4)) * QLD, m, n, A);
             }
           }
           __syncthreads();
@@ -334,7 +523,7 @@ k_jacobi32(Pre32 a, unsigned int* st) {
           Ga = Gb;
           Gb = t;
         }
-        if (tid < PB) atomicMax(&s_off, __float_as_int(off));
+        if (warp == 4 && lane < PB) atomicMax(&s_off, __float_as_int(off));
         // ---- heavier rows first
         if (tid < PM) {
           const float di = Ga[tid * GLD + tid].x;
@@ -356,49 +545,29 @@ k_jacobi32(Pre32 a, unsigned int* st) {
             stage(u, v, c0, n);
             __syncthreads();
           }
-          for (int cb = (warp >> 2) * 32; cb < n; cb += 64) {
-            const int c = cb + lane;
-            const bool in = c < n;
-            const float2* sp = S + (in ? c : 0);
-            float2 o[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) o[i] = make_float2(0.f, 0.f);
-#pragma unroll 8
-            for (int m = 0; m < PM; ++m) {
-              const float2 s = sp[m * ld];
-              const float4* qp = reinterpret_cast<const float4*>(QT + m * QLD + r0);
-#pragma unroll
-              for (int i2 = 0; i2 < 4; ++i2) {
-                const float4 q = qp[i2];
-                float2& o0 = o[2 * i2];
-                float2& o1 = o[2 * i2 + 1];
-                o0.x = fmaf(q.x, s.x, fmaf(-q.y, s.y, o0.x));
-                o0.y = fmaf(q.x, s.y, fmaf(q.y, s.x, o0.y));
-                o1.x = fmaf(q.z, s.x, fmaf(-q.w, s.y, o1.x));
-                o1.y = fmaf(q.z, s.y, fmaf(q.w, s.x, o1.y));
-              }
-            }
-            if (in) {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const int pos = s_pos[r0 + i];
-                const int row = pos < PB ? u * PB + pos : v * PB + pos - PB;
-                *reinterpret_cast<float2*>(col_ptr(a, row, rank, c0 + c)) = o[i];
-              }
-            }
+          // a lane takes 1 to 4 columns 64 apart, so that the reads of Q are
+          // shared by as many products as the chunk has
+          for (int cb = 0; cb < n; cb += 256) {
+            const int left = n - cb;
+            if (left > 192) apply_rows<4>(a, S, QT, s_pos, ld, cb, n, r0, u, v, rank, c0);
+            else if (left > 128) apply_rows<3>(a, S, QT, s_pos, ld, cb, n, r0, u, v, rank, c0);
+            else if (left > 64) apply_rows<2>(a, S, QT, s_pos, ld, cb, n, r0, u, v, rank, c0);
+            else apply_rows<1>(a, S, QT, s_pos, ld, cb, n, r0, u, v, rank, c0);
           }
         }
-        // a further pair of this cluster overwrites part, read by the others
-        cl.sync();
+        __syncthreads();
+        if (tid == 0) {
+          publish_block(a.ver + u * 8 + rank, step + 1);
+          publish_block(a.ver + v * 8 + rank, step + 1);
+        }
       }
-      cl.sync();
-      passed += (unsigned int)ncl;
-      if (rank == 0 && tid == 0) s_ok = leader_barrier(st, passed) ? 1 : 0;
-      cl.sync();
-      ok = *cl.map_shared_rank(&s_ok, 0) != 0;
-      if (!ok) break;
     }
-    if (!ok) break;
+    // ---- every block has been through the sweep
+    cl.sync();
+    passed += (unsigned int)ncl;
+    if (rank == 0 && tid == 0) s_ok = leader_barrier(st, passed) ? 1 : 0;
+    cl.sync();
+    if (*cl.map_shared_rank(&s_ok, 0) == 0) break;
     if (blockIdx.x == 0 && tid == 0) st[C_SWEEPS] = (unsigned int)(sw + 1);
     if (__int_as_float((int)__ldcg(st + C_OFF + sw)) <= kStop32) break;
   }
@@ -629,9 +798,11 @@ PreDims pre_dims(int k, int p) {
   const int kp = (int)round_up(k, PM);
   return {kp, (int)round_up(p, 4) + 32, kp + 32};
 }
+// control words, then the blocks' step counts
+size_t ctl_bytes(const PreDims& d) { return (size_t)(C_WORDS + d.kp / PB * 8) * sizeof(int); }
 int share(int columns, int C) { return 4 * ((columns + 4 * C - 1) / (4 * C)); }
 
-constexpr size_t kFixedSmem = (size_t)PM * (3 * GLD + QLD) * sizeof(float2);
+constexpr size_t kFixedSmem = (size_t)PM * (4 * GLD + QLD) * sizeof(float2);
 constexpr int kChunkMax = 640;                // columns staged at once: 32 x 642 x 8 B = 164 KB
 constexpr size_t kOwnSmSmem = 116 * 1024;     // more than half of an SM's shared memory
 
@@ -688,7 +859,7 @@ cudaError_t cluster_capacity(int C, size_t smem, int* n) {
 size_t svd_pre_bytes(int k, int p) {
   const PreDims d = pre_dims(k, p);
   return (size_t)d.kp * (d.pl + d.vl) * sizeof(float2) + 4 * (size_t)k * k * sizeof(cplx) +
-         (size_t)(2 * k + 1) * sizeof(int) + C_WORDS * sizeof(int) + 6 * 256;
+         (size_t)(2 * k + 1) * sizeof(int) + ctl_bytes(d) + 6 * 256;
 }
 
 SvdPre svd_pre_carve(void* ws, int k, int p) {
@@ -703,7 +874,7 @@ SvdPre svd_pre_carve(void* ws, int k, int p) {
   s.rows32 = take((size_t)d.kp * (d.pl + d.vl) * sizeof(float2));
   for (cplx*& m : s.K) m = reinterpret_cast<cplx*>(take((size_t)k * k * sizeof(cplx)));
   s.act = reinterpret_cast<int*>(take((size_t)(2 * k + 1) * sizeof(int)));
-  s.ctl = reinterpret_cast<unsigned int*>(take(C_WORDS * sizeof(int)));
+  s.ctl = reinterpret_cast<unsigned int*>(take(ctl_bytes(d)));
   s.ok = reinterpret_cast<int*>(s.ctl + C_OK);
   s.gate_n = reinterpret_cast<int*>(s.ctl + C_GN);
   s.gate = reinterpret_cast<int*>(s.ctl + C_GE);
@@ -716,7 +887,7 @@ SvdPre svd_pre_carve(void* ws, int k, int p) {
 cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const double* anorm2,
                            cudaStream_t st) {
   const PreDims d = pre_dims(k, p);
-  cudaError_t err = cudaMemsetAsync(s.ctl, 0, C_WORDS * sizeof(int), st);
+  cudaError_t err = cudaMemsetAsync(s.ctl, 0, ctl_bytes(d), st);
   if (err != cudaSuccess) return err;
   Pre32 a;
   a.R = static_cast<float2*>(s.rows32);
@@ -726,6 +897,7 @@ cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const d
   a.pl = d.pl;
   a.vl = d.vl;
   a.nb = d.kp / PB;
+  a.ver = s.ctl + C_WORDS;
   count_launches(1);
   k_pre_init<<<grid_for((long long)d.kp * (d.pl + d.vl)), 256, 0, st>>>(R, p, anorm2, a);
   // as many CTAs per pair as give every CTA an SM of its own (two on one SM

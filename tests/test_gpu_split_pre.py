@@ -78,6 +78,21 @@ def test_split_against_svd(api, ctx, m, n, kind):
         assert abs(disc - disc_ref) <= 1e-10 * max(disc_ref, 1e-12) + 1e-15
 
 
+@pytest.mark.parametrize("seed", range(8))
+def test_rows_of_very_different_weight_stay_preconditioned(api, ctx, seed):
+    # squared norms down to 1e-26 of the largest: a rotation between a heavy and a
+    # light row has to stay unitary, or all rows go to the FP64 Jacobi; left to it
+    # are only members of groups of equal values, so it does less than the inner
+    # products (8 flops a term) of one sweep over all pairs
+    m, n = 274, 366
+    X = _matrix(np.random.default_rng(seed), m, n, "groups")
+    api.svd_stats(ctx)
+    _split(api, ctx, X, 200, 1e-10, False, True)
+    st = api.svd_stats(ctx)
+    assert st["splits"] == 1
+    assert st["jacobi_fp64_flops"] < m * (m - 1) / 2 * 8 * m
+
+
 @pytest.mark.parametrize("scale", [1e-60, 1e60])
 def test_split_is_invariant_under_scaling(api, ctx, scale):
     X = _matrix(np.random.default_rng(3), 70, 90, "decay")
