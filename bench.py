@@ -41,13 +41,15 @@ UNIT = "tau-steps/s"
 # 2 DFMA/clk x 2 FLOP x 2.07 GHz = 1.26 TFLOP/s, in line with the nominal
 # 1.25 TFLOP/s (a DFMA probe measured 1.19 at 1995 MHz).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# DRAM bytes (read + write) of one k_jacobi_persistent launch on the bulk
-# 512 x 512 split from the ncu capture of this kernel source summarised in
-# profiles/k_jacobi_persistent_split512.md (None once the kernel changes).
-JACOBI_TRAFFIC_BYTES = 4.268544e6 + 1.094656e6
-JACOBI_TRAFFIC_NOTE = ("dram bytes per launch on the 512 x 512 bulk split (ncu, "
-                       "profiles/k_jacobi_persistent_split512.md); the matrix is L2-resident, "
-                       "the kernel is FP64-bound")
+# FP32 pipe: 152 SMs x 128 FMA/clk x 2 FLOP x 2.07 GHz, derived likewise
+FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
+# Compulsory bytes of one k_jacobi32 launch on the bulk 512 x 512 split: R and V
+# (512 x 512 complex64 each) read and written once
+JACOBI_TRAFFIC_BYTES = 2 * 2 * 512 * 512 * 8
+JACOBI_TRAFFIC_NOTE = ("R and V of one 512 x 512 split read and written once, by count (the "
+                       "profiler does not keep the kernel's cluster launch, "
+                       "profiles/k_jacobi32_split512.md); both are L2-resident, the kernel is "
+                       "bound by its chain of dependent rounds")
 WORKLOAD = ("heisenberg_bulk: XXX chain N=64 J=1 OBC, D=5, chi_max=256, cutoff 1e-10, "
             "backward Euler on geometric grid 1e-3->1e3 (40 steps), shift=current energy, "
             "saturated synthetic start (chi=256 bulk)")
@@ -590,21 +592,24 @@ def run_ours(args, rank, world, local_rank):
                     "d2h_bytes_per_step": hio.d2h // args.steps,
                     "same_steps_as_value": True, "same_energies_as_value": e2e_same},
             "gpu_launches": int(launches),
-            "roofline": {"kernel": "k_jacobi_persistent (one-sided Jacobi of the SVD splits)",
-                         "bound": "alu", "achieved": jac_tf, "peak": FP64_PEAK_TFLOPS,
-                         "unit": "TFLOP/s", "frac": jac_tf / FP64_PEAK_TFLOPS,
+            "roofline": {"kernel": ("Jacobi stage of the SVD splits (k_jacobi32 in fp32, FP64-class "
+                                    "corrections, k_jacobi_persistent on the rows left)"),
+                         "bound": "latency", "achieved": jac_tf, "peak": FP32_PEAK_TFLOPS,
+                         "unit": "TFLOP/s", "frac": jac_tf / FP32_PEAK_TFLOPS,
+                         "frac_of_fp64_pipe": jac_tf / FP64_PEAK_TFLOPS,
                          "traffic": JACOBI_TRAFFIC_BYTES,
                          "traffic_note": JACOBI_TRAFFIC_NOTE,
                          "achieved_note": ("algorithmic SVD work (22 n^3-class count: 8.7 GFLOP "
                                            "per 512 x 512 split, scaled by m n min(m,n)) over "
-                                           "the Jacobi kernel's CUDA-event time"),
+                                           "the stage's CUDA-event time"),
                          "device_counted_tflops": jac_dev_tf,
                          "launches": jac["count"], "ms_per_launch": jac["ms"] / max(1, jac["count"]),
-                         "peak_note": ("derived, not measured: FP64 pipe from unit counts and "
-                                       "clocks (152 SMs x 4 FLOP/clk x 2.07 GHz)"),
+                         "peak_note": ("derived, not measured: FP32 pipe from unit counts and "
+                                       "clocks (152 SMs x 256 FLOP/clk x 2.07 GHz); the "
+                                       "device-counted FLOPs are those of the FP64 kernel"),
                          "share_of_step": jac["ms"] / max(1e-9, prof["step"]["ms"])},
             "roofline_other": {
-                "lq": {"kernel": "k_lq_persistent (Householder LQ of the SVD splits)", "bound": "alu",
+                "lq": {"kernel": "k_lq_resident (Householder LQ of the SVD splits)", "bound": "alu",
                        "achieved": lq_tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                        "frac": lq_tf / FP64_PEAK_TFLOPS,
                        "share_of_step": lq["ms"] / max(1e-9, prof["step"]["ms"])},

@@ -46,10 +46,9 @@ constexpr int kJacobiSweeps = 30;
 constexpr int kMaxKrylov = 32;
 constexpr double kEmuMinWork = 2.0e6;    // complex MACs below which GEMMs stay native
 // Rows from which the Jacobi of a split is preconditioned.  A whole split of k x k,
-// without and with it: k = 16 0.81 and 0.70 ms, 24 1.36 and 0.91, 32 2.00 and
-// 1.05, 64 4.36 and 1.80, 512 69.9 and 13.9.  Below 16 rows
-// one cluster step covers the whole matrix and the GEMMs' launches outweigh the
-// few rounds saved.
+// without and with it: k = 16 0.84 and 0.44 ms, 24 1.43 and 0.47, 32 1.91 and
+// 0.50, 64 4.20 and 0.87, 512 69 and 9.0.  Below 16 rows one block pair is
+// mostly padding (12 rows take 0.59 ms without).
 constexpr int kPreMinRows = 16;
 // Algorithmic FP64 work of a truncated SVD of a p x q complex block, as the
 // reference count that roofline figures divide by: the 22 n^3-class estimate

@@ -4,13 +4,17 @@
 // side whose isometry is wanted, the split runs
 //   1. a Householder LQ of the rows, Xr H_0 H_1 ... H_{k-1} = L (p x k lower
 //      trapezoidal, k = min(p, q)), all k reflector steps in one cooperative
-//      launch;
+//      launch: k_lq_resident holds the rows in registers or shared memory,
+//      k_lq_persistent is for rows that fit in neither;
 //   2. R = L^H (k x p, upper trapezoidal), so that R^H R = Xr Xr^H: the rows
 //      of R carry the left singular structure of Xr and are graded like its
 //      singular values, which is what lets the Jacobi below converge in few
 //      sweeps (QR preconditioning of the one-sided Jacobi method);
-//   3. one-sided (Hestenes) Jacobi on the rows of R until they are mutually
-//      orthogonal: R_out = Sigma U^H, U the left singular vectors of Xr;
+//   3. from 16 rows the preconditioner of svd_pre.cu, which leaves the rows of
+//      R orthogonal up to members of near-degenerate groups, then one-sided
+//      (Hestenes) FP64 Jacobi on the rows it lists (on all rows without it)
+//      until they are mutually orthogonal: R_out = Sigma U^H, U the left
+//      singular vectors of Xr;
 //   4. row norms, the descending order and the truncation rule; the kept
 //      rows of U^H are the rows of R_out divided by their norms.
 // No rotation is accumulated: the engine forms the other factor as the
