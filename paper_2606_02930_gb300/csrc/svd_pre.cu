@@ -291,7 +291,7 @@ __device__ __forceinline__ void apply_rows(const Pre32& a, const float2* S, cons
 // Bound: latency and shared memory.  Clocks per step at k = 512 (16 pairs, 6 CTAs
 // each, 31 steps a sweep): wait for the blocks 1.7k, copy in 1.7k, Gram 4.3k, sum
 // 3.3k, the 16 or 31 dependent rounds 13.8k (620 each: the chain of approximate
-// square roots on warp 4), rows 12k; 19 us in all.  With a barrier over the grid
+// square roots on warp 4), rows 11k; 19 us in all.  With a barrier over the grid
 // after every step, the rotations formed before the update and 2 x 2 tiles in the
 // Gram matrix: 23.7 us.  16-row blocks: 8-row ones need twice the steps for the
 // same number of rounds, 32-row ones leave half the SMs without a pair.  Whole
