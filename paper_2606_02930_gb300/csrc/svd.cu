@@ -169,7 +169,7 @@ k_lq_persistent(cplx* W, int p, int q, cplx* beta, double* refl, unsigned int* s
 // Polls are bounded; a block that gives up sets the error word, which the others
 // see in their own polls, and leaves.
 // Measured, with the barrier kernel above before: 64 x 64 0.41 -> 0.26 ms, 512 x 512
-// 6.4 -> 2.7, 1024 x 1024 25.7 -> 11.6 (5.3 us a step at 512: about 1 us from store
+// 6.4 -> 2.65, 1024 x 1024 25.7 -> 11.5 (5.2 us a step at 512: about 1 us from store
 // to load, the rest the FP64 chain of the next pivot row; at 1024 the seven rows a
 // block holds).
 constexpr int LT = 128;                       // threads
@@ -209,24 +209,6 @@ __device__ __forceinline__ double warp_sum8(double (&v)[8]) {
   r += __shfl_xor_sync(0xffffffffu, r, 2);
   r += __shfl_xor_sync(0xffffffffu, r, 1);
   return r;
-}
-
-constexpr double kTinySq = 1e-280, kHugeSq = 1e280;   // range of the two functions below
-
-// 1 / sqrt(x) and 1 / x for x in that range from the hardware's approximations
-// (about 20 bits) and one step of third order each, e = 1 - x y^2 (or 1 - x y):
-// y (1 + e / 2 + 3 e^2 / 8) and y (1 + e + e^2), to about an ulp.
-__device__ __forceinline__ double rsqrt_fp64(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y * e, fma(e, 0.375, 0.5), y);
-}
-__device__ __forceinline__ double rcp_fp64(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
 }
 
 // One element of a row per thread and LT columns: EPT >= q / LT
@@ -321,16 +303,14 @@ k_lq_resident(cplx* W, int p, int q, cplx* beta, double* refl, cplx* pub, unsign
           // u_0 = x_0 (1 + |x| / |x_0|), c = 1 / (|x|^2 + |x| |x_0|)
           const cplx x0 = s_x0;
           if (lane == 7) t = fma(x0.x, x0.x, x0.y * x0.y);
-          double rs = 0.0;
-          if (t > kTinySq && t < kHugeSq) rs = rsqrt_fp64(t);
-          else if (t > 0.0) rs = rsqrt(t);
+          const double rs = t > 0.0 ? rsqrt(t) : 0.0;
           const double n2 = __shfl_sync(0xffffffffu, t, 6);
           const double a2 = __shfl_sync(0xffffffffu, t, 7), ra = __shfl_sync(0xffffffffu, rs, 7);
           const double nx = n2 * __shfl_sync(0xffffffffu, rs, 6);
           const double g = nx * ra;
           const cplx du = a2 > 0.0 ? cmake(x0.x * g, x0.y * g) : cmake(nx, 0.0);   // u_0 - x_0
           const double den = fma(nx, a2 * ra, n2);
-          const double c = den > kTinySq && den < kHugeSq ? rcp_fp64(den) : n2 > 0.0 ? 1.0 / den : 0.0;
+          const double c = n2 > 0.0 ? 1.0 / den : 0.0;
           if (lane == 0) {
             s_c = c;
             s_du = du;
