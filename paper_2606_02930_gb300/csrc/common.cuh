@@ -51,6 +51,9 @@ struct GemmArgs {
   cplx alpha, beta;
   const cplx* Z; cplx gamma;   // optional: C = alpha*AB + beta*C + gamma*Z
   const int* run_if = nullptr; // optional device word: nothing is computed when it is 0
+  // optional, K device words: zgemm_emu multiplies column k of A by 2^kexp[k] and
+  // row k of B by 2^-kexp[k] as it cuts them (exact); zgemm has no use for them
+  const int* kexp = nullptr;
 };
 cudaError_t zgemm(const GemmArgs& g, cudaStream_t st);
 
@@ -220,17 +223,18 @@ struct SvdPre {
   void* rows32;
   cplx* K[4];
   int *act, *ok, *gate_n, *gate, *gate_w, *gate_w2, *err;
+  int* rexp;                   // powers of two next to the row norms, for GemmArgs::kexp
   unsigned int* ctl;
 };
 size_t svd_pre_bytes(int k, int p);
 SvdPre svd_pre_carve(void* ws, int k, int p);
-// K[0] = V (k x k) from the fp32 block Jacobi on the rows of R; clears the
-// control words.  One cooperative launch of clusters.
+// K[0] = V (k x k) from the fp32 block Jacobi on the rows of R, rexp from R; clears
+// the control words.  One cooperative launch of clusters.
 cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const double* anorm2,
                            cudaStream_t st);
 // M = V V^H (k x k) becomes -(M - I) / 2; step 0 decides *ok, step 1 *gate_n
 cudaError_t svd_pre_orth(const SvdPre& s, cplx* M, int k, int step, cudaStream_t st);
-// E (k x k) from G = S S^H, and the gates
+// E (k x k) and rexp from G = S S^H, and the gates
 cudaError_t svd_pre_corr(const SvdPre& s, const cplx* G, int k, double tol, const double* anorm2,
                          double skip_rel, cplx* E, cudaStream_t st);
 // E += W / 2 - W2 / 8 as the gates say

@@ -284,9 +284,10 @@ ite_status gemm(ite_ctx ctx, int M, int N, int K, const cplx* A, long long sAm, 
                 bool conjA, const cplx* B, long long sBk, long long sBn, bool conjB, cplx* Cm,
                 long long ldc, cplx alpha = C(1), cplx beta = C(0), const cplx* Z = nullptr,
                 cplx gamma = C(0), int batch = 1, long long sAb = 0, long long sBb = 0,
-                long long sCb = 0, const int* run_if = nullptr) {
+                long long sCb = 0, const int* run_if = nullptr, const int* kexp = nullptr) {
   GemmArgs g;
   g.run_if = run_if;
+  g.kexp = kexp;
   g.M = M; g.N = N; g.K = K; g.batch = batch;
   g.A = A; g.sAm = sAm; g.sAk = sAk; g.sAb = sAb; g.conjA = conjA;
   g.B = B; g.sBk = sBk; g.sBn = sBn; g.sBb = sBb; g.conjB = conjB;
@@ -455,13 +456,14 @@ ite_status merge(ite_ctx ctx, int d, int chl, int chm, int chr, const cplx* K1, 
               (long long)d * chr);
 }
 
-// Y += D Y (D k x k, Y k x len) unless *run_if is 0; tmp holds k x len.  The
-// emulated GEMM reads Y only while slicing it, so it works in place.
+// Y += D Y (D k x k, Y k x len) unless *run_if is 0; tmp holds k x len, rexp the
+// powers of two next to the norms of Y's rows (unit rows without).  The emulated
+// GEMM reads Y only while slicing it, so it works in place.
 ite_status add_left(ite_ctx ctx, const cplx* D, cplx* Y, int k, int len, cplx* tmp,
-                    const int* run_if) {
+                    const int* run_if, const int* rexp = nullptr) {
   if (emulated(ctx, k, len, k))
     return gemm(ctx, k, len, k, D, k, 1, false, Y, len, 1, false, Y, len, C(1), C(1), nullptr, C(0),
-                1, 0, 0, 0, run_if);
+                1, 0, 0, 0, run_if, rexp);
   CS(gemm(ctx, k, len, k, D, k, 1, false, Y, len, 1, false, tmp, len, C(1), C(0), Y, C(1), 1, 0, 0,
           0, run_if));
   CK(vec_copy_if(Y, tmp, (long long)k * len, run_if, true, ctx->stream));
@@ -488,7 +490,7 @@ ite_status precondition(ite_ctx ctx, cplx* R, cplx* S, int k, int p, const doubl
     CS(add_left(ctx, B, A, k, k, W, it == 0 ? s.ok : on));
   }
   CS(gemm(ctx, k, p, k, A, k, 1, false, R, p, 1, false, S, p, C(1), C(0), nullptr, C(0), 1, 0, 0, 0,
-          s.ok));
+          s.ok, s.rexp));
   CK(vec_copy_if(S, R, (long long)k * p, s.ok, false, ctx->stream));
   for (int it = 0; it < 2; ++it) {
     CS(gram(S, p, B));
@@ -498,7 +500,7 @@ ite_status precondition(ite_ctx ctx, cplx* R, cplx* S, int k, int p, const doubl
     CS(gemm(ctx, k, k, k, W, k, 1, false, W, k, 1, false, W2, k, C(1), C(0), nullptr, C(0), 1, 0, 0,
             0, s.gate_w2));
     CK(svd_pre_comb(s, A, W, W2, k, ctx->stream));
-    CS(add_left(ctx, A, S, k, p, R, s.gate));
+    CS(add_left(ctx, A, S, k, p, R, s.gate, s.rexp));
   }
   CS(gram(S, p, B));
   CK(svd_pre_list(s, B, k, tol, anorm2, skip_rel, ctx->stream));

@@ -21,10 +21,16 @@
 //      Jacobi's tolerance (members of near-degenerate groups, or all rows if
 //      a check below failed); the FP64 Jacobi runs on those rows only.
 // Every transformation applied is unitary to FP64 rounding, and the FP64
-// Jacobi's criterion decides what remains, so the factors are as accurate as
-// without the preconditioner.  S is updated by small corrections D S rather
-// than replaced by Q S so that the light rows keep their relative accuracy:
-// the FP64-class GEMM's error is relative to the largest entry of D's row.
+// Jacobi's criterion decides what remains.  Rows of very different weight: an
+// FP64-class product is accurate relative to the largest entry of a row of its
+// left and of a column of its right factor, so V R and D S alone would leave the
+// light rows an error of 2^-56 of the heaviest (a singular value of 1e-10 of the
+// largest was off by 3e-8 of itself, for 300 rows graded along the columns).  The
+// rows of R and S are therefore divided by the powers of two next to their norms,
+// and the columns of V and D multiplied by them (rexp, exact, while the operands are
+// cut): the entries of (V diag d)_i are then what the terms of row i weigh, and the
+// singular values keep the relative accuracy of FP64 products (1e-15 in that case).
+// S is updated by small corrections D S rather than replaced by Q S.
 // Guards: V is dropped (S = R, all rows go to the Jacobi) unless
 // |V V^H - I|_inf < 1e-2, from which three Newton-Schulz steps reach rounding;
 // a correction is dropped unless |E|_inf <= 2e-3.
@@ -574,24 +580,38 @@ k_jacobi32(Pre32 a, unsigned int* st) {
   cl.sync();                    // s_ok of the first CTA stays readable until here
 }
 
-// R32 = R / |R|_F with zero padding, V = I
-__global__ void k_pre_init(const cplx* __restrict__ R, int p, const double* anorm2, Pre32 a) {
+constexpr int RT = 128;                       // threads of the row kernels
+
+// Row i of R32 = R / |R|_F with zero padding, of V = I, and rexp[i] with
+// 2^rexp[i] above the largest entry of row i of R, at most twice it.
+__global__ void __launch_bounds__(RT)
+k_pre_init(const cplx* __restrict__ R, int p, const double* anorm2, Pre32 a, int* rexp) {
   const double n2 = *anorm2;
   const double s = n2 > 0.0 && isfinite(n2) ? rsqrt(n2) : 0.0;
-  const long long w = a.pl + a.vl, tot = w * a.kp;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
-       e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e / w), c = (int)(e - (long long)i * w);
-    if (c < a.pl) {
-      float2 v = make_float2(0.f, 0.f);
-      if (i < a.k && c < p) {
-        const cplx x = R[(long long)i * p + c];
-        v = make_float2((float)(x.x * s), (float)(x.y * s));
-      }
-      a.R[(long long)i * a.pl + c] = v;
-    } else {
-      a.V[(long long)i * a.vl + c - a.pl] = make_float2(i == c - a.pl ? 1.f : 0.f, 0.f);
+  const int i = blockIdx.x;
+  unsigned long long mx = 0ull;
+  for (int c = threadIdx.x; c < a.pl; c += RT) {
+    float2 v = make_float2(0.f, 0.f);
+    if (i < a.k && c < p) {
+      const cplx x = R[(long long)i * p + c];
+      v = make_float2((float)(x.x * s), (float)(x.y * s));
+      mx = max(mx, (unsigned long long)__double_as_longlong(fmax(fabs(x.x), fabs(x.y))));
     }
+    a.R[(long long)i * a.pl + c] = v;
+  }
+  for (int c = threadIdx.x; c < a.vl; c += RT)
+    a.V[(long long)i * a.vl + c] = make_float2(i == c ? 1.f : 0.f, 0.f);
+  if (i >= a.k) return;
+  // the exponent field of the largest magnitude orders like it
+  const int e = __reduce_max_sync(0xffffffffu, (int)(mx >> 52));
+  __shared__ int sh[RT / 32];
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = e;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int m = 0;
+#pragma unroll
+    for (int w = 0; w < RT / 32; ++w) m = max(m, sh[w]);
+    rexp[i] = m == 0 ? 0 : m - 1022;
   }
 }
 
@@ -604,8 +624,6 @@ __global__ void k_pre_export(Pre32 a, cplx* __restrict__ V) {
     V[e] = cmake(v.x, v.y);
   }
 }
-
-constexpr int RT = 128;                       // threads of the row kernels
 
 __device__ __forceinline__ double block_sum(double v) {
   __shared__ double sh[RT / 32];
@@ -676,14 +694,17 @@ constexpr double kNuMax = 2e-3;
 
 // E from G = S S^H: E_ij = -sign(D) t g_ij / |g_ij| (D = G_jj - G_ii, t the tangent of
 // the rotation that makes the pair orthogonal), exactly anti-Hermitian because
-// both halves come from the upper triangle.  The last block sets the gates of
-// what follows from nu = |E|_inf: E^2 counts above 4e-9, E^4 above 1e-4.
+// both halves come from the upper triangle; rexp[i] with 2^rexp[i] next to |S_i|.
+// The last block sets the gates of what follows from nu = |E|_inf: E^2 counts above
+// 4e-9, E^4 above 1e-4.
 __global__ void __launch_bounds__(RT)
 k_pre_corr(const cplx* __restrict__ G, int k, double tol, const double* anorm2, double skip_rel,
-           cplx* __restrict__ E, unsigned int* ctl) {
+           cplx* __restrict__ E, int* rexp, unsigned int* ctl) {
   const int i = blockIdx.x;
   const double skip = skip_rel * *anorm2;
   const double al = G[(long long)i * k + i].x;
+  if (threadIdx.x == 0)
+    rexp[i] = al > 0.0 ? (((int)((unsigned long long)__double_as_longlong(al) >> 52) - 1023) >> 1) + 1 : 0;
   double s = 0.0;
   for (int j = threadIdx.x; j < k; j += RT) {
     cplx e = cmake(0.0, 0.0);
@@ -859,7 +880,7 @@ cudaError_t cluster_capacity(int C, size_t smem, int* n) {
 size_t svd_pre_bytes(int k, int p) {
   const PreDims d = pre_dims(k, p);
   return (size_t)d.kp * (d.pl + d.vl) * sizeof(float2) + 4 * (size_t)k * k * sizeof(cplx) +
-         (size_t)(2 * k + 1) * sizeof(int) + ctl_bytes(d) + 6 * 256;
+         (size_t)(3 * k + 1) * sizeof(int) + ctl_bytes(d) + 6 * 256;
 }
 
 SvdPre svd_pre_carve(void* ws, int k, int p) {
@@ -873,7 +894,8 @@ SvdPre svd_pre_carve(void* ws, int k, int p) {
   };
   s.rows32 = take((size_t)d.kp * (d.pl + d.vl) * sizeof(float2));
   for (cplx*& m : s.K) m = reinterpret_cast<cplx*>(take((size_t)k * k * sizeof(cplx)));
-  s.act = reinterpret_cast<int*>(take((size_t)(2 * k + 1) * sizeof(int)));
+  s.act = reinterpret_cast<int*>(take((size_t)(3 * k + 1) * sizeof(int)));
+  s.rexp = s.act + 2 * k + 1;
   s.ctl = reinterpret_cast<unsigned int*>(take(ctl_bytes(d)));
   s.ok = reinterpret_cast<int*>(s.ctl + C_OK);
   s.gate_n = reinterpret_cast<int*>(s.ctl + C_GN);
@@ -899,7 +921,7 @@ cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const d
   a.nb = d.kp / PB;
   a.ver = s.ctl + C_WORDS;
   count_launches(1);
-  k_pre_init<<<grid_for((long long)d.kp * (d.pl + d.vl)), 256, 0, st>>>(R, p, anorm2, a);
+  k_pre_init<<<d.kp, RT, 0, st>>>(R, p, anorm2, a, s.rexp);
   // as many CTAs per pair as give every CTA an SM of its own (two on one SM
   // take turns at every phase of the step)
   const int pairs = a.nb / 2;
@@ -945,7 +967,7 @@ cudaError_t vec_copy_if(cplx* y, const cplx* x, long long n, const int* flag, bo
 cudaError_t svd_pre_corr(const SvdPre& s, const cplx* G, int k, double tol, const double* anorm2,
                          double skip_rel, cplx* E, cudaStream_t st) {
   count_launches(1);
-  k_pre_corr<<<k, RT, 0, st>>>(G, k, tol, anorm2, skip_rel, E, s.ctl);
+  k_pre_corr<<<k, RT, 0, st>>>(G, k, tol, anorm2, skip_rel, E, s.rexp, s.ctl);
   return cudaGetLastError();
 }
 

@@ -412,7 +412,32 @@ struct Operand {
   int conj, rows, nb;
   __nv_bfloat16* out;                           // digits: (digit, batch, real row, K)
   int* e;                                       // exponents: (batch, row)
+  const int* kexp;                              // entry k times 2^(ksign kexp[k])
+  int ksign;
 };
+
+// x 2^d by its exponent field (exact; what leaves the normal range at the lower
+// end is 0)
+__device__ __forceinline__ double shifted(double x, int d) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int E = (int)(b >> 52) & 0x7FF, to = E + d;
+  if (E == 0 || E == 0x7FF) return x;
+  if (to < 1) return 0.0;
+  return __longlong_as_double((long long)((b & 0x800FFFFFFFFFFFFFull) |
+                                          (unsigned long long)min(to, 0x7FE) << 52));
+}
+
+// entry k of the row of `o` that starts at x (SCALED: kexp counts; an instance of its
+// own, because the test alone cost the H_eff's cuts a fifth of their time)
+template <bool SCALED>
+__device__ __forceinline__ cplx entry(const Operand& o, const cplx* x, int k) {
+  cplx v = x[(long long)k * o.sk];
+  if (SCALED) {
+    const int d = o.ksign * o.kexp[k];
+    v = cmake(shifted(v.x, d), shifted(v.y, d));
+  }
+  return v;
+}
 
 constexpr int CR = 8;                           // rows per block
 
@@ -445,7 +470,7 @@ __device__ __forceinline__ void write_digits(const Operand& o, long long row, lo
 // time and turned through shared memory, so that both kinds read whole sectors
 // and write 128-byte runs.  (One warp per row reading a column with stride took 34 us
 // for the 256 columns of 1280 entries of a chi = 256 H_eff.)
-template <bool EMBED>
+template <bool EMBED, bool SCALED>
 __device__ void cut_rows(const Operand& o, int blk, int K, int Kp) {
   __shared__ unsigned long long smax[8][CR];
   __shared__ cplx tile[CR][129];
@@ -463,7 +488,7 @@ __device__ void cut_rows(const Operand& o, int blk, int K, int Kp) {
     unsigned long long mx = 0;
 #pragma unroll 4
     for (int k = lane; k < K; k += 32) {
-      const cplx v = x[(long long)k * o.sk];
+      const cplx v = entry<SCALED>(o, x, k);
       mx = max(mx, max(mag_bits(v.x), mag_bits(v.y)));
     }
 #pragma unroll
@@ -472,7 +497,7 @@ __device__ void cut_rows(const Operand& o, int blk, int K, int Kp) {
     if (lane == 0) o.e[b * o.rows + r] = e;
     for (int k = lane; k < Kc; k += 32)
       write_digits<EMBED>(o, row, digit_stride, Kp, k,
-                          k < K ? x[(long long)k * o.sk] : cmake(0.0, 0.0), e);
+                          k < K ? entry<SCALED>(o, x, k) : cmake(0.0, 0.0), e);
     return;
   }
   const int tr = tid & (CR - 1), tk = tid / CR;              // 32 entries of K at a time
@@ -482,7 +507,7 @@ __device__ void cut_rows(const Operand& o, int blk, int K, int Kp) {
   if (in) {
 #pragma unroll 4
     for (int k = tk; k < K; k += 32) {
-      const cplx v = x[(long long)k * o.sk];
+      const cplx v = entry<SCALED>(o, x, k);
       mx = max(mx, max(mag_bits(v.x), mag_bits(v.y)));
     }
   }
@@ -500,7 +525,7 @@ __device__ void cut_rows(const Operand& o, int blk, int K, int Kp) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       const int k = k0 + tk + 32 * i;
-      tile[tr][tk + 32 * i] = in && k < K ? x[(long long)k * o.sk] : cmake(0.0, 0.0);
+      tile[tr][tk + 32 * i] = in && k < K ? entry<SCALED>(o, x, k) : cmake(0.0, 0.0);
     }
     __syncthreads();
     if (r < o.rows) {
@@ -513,11 +538,12 @@ __device__ void cut_rows(const Operand& o, int blk, int K, int Kp) {
   }
 }
 
+template <bool SCALED>
 __global__ void __launch_bounds__(256)
 k_cut_digits(Operand A, Operand B, int K, int Kp, int blocksA, const int* run_if) {
   if (run_if && *run_if == 0) return;
-  if ((int)blockIdx.x < blocksA) cut_rows<true>(A, blockIdx.x, K, Kp);
-  else cut_rows<false>(B, blockIdx.x - blocksA, K, Kp);
+  if ((int)blockIdx.x < blocksA) cut_rows<true, SCALED>(A, blockIdx.x, K, Kp);
+  else cut_rows<false, SCALED>(B, blockIdx.x - blocksA, K, Kp);
 }
 
 long long padded_k(int K) { return ((2LL * (K > 0 ? K : 1) + BK - 1) / BK) * BK; }
@@ -584,11 +610,16 @@ cudaError_t zgemm_emu(const GemmArgs& g, void* scratch, size_t scratch_bytes, in
     if (e != cudaSuccess) return e;
     sm_count[dev & 63].store(sms);
   }
-  const Operand oA = {g.A, g.sAm, g.sAk, g.sAb, g.conjA ? 1 : 0, g.M, nbA, As, eA};
-  const Operand oB = {g.B, g.sBn, g.sBk, g.sBb, g.conjB ? 1 : 0, g.N, nbB, Bs, eB};
+  const Operand oA = {g.A, g.sAm, g.sAk, g.sAb, g.conjA ? 1 : 0, g.M, nbA, As, eA,
+                      g.kexp, 1};
+  const Operand oB = {g.B, g.sBn, g.sBk, g.sBb, g.conjB ? 1 : 0, g.N, nbB, Bs, eB,
+                      g.kexp, -1};
   const int blocksA = (g.M + CR - 1) / CR * nbA, blocksB = (g.N + CR - 1) / CR * nbB;
   count_launches(1);
-  k_cut_digits<<<blocksA + blocksB, 256, 0, st>>>(oA, oB, g.K, (int)Kp, blocksA, g.run_if);
+  if (g.kexp)
+    k_cut_digits<true><<<blocksA + blocksB, 256, 0, st>>>(oA, oB, g.K, (int)Kp, blocksA, g.run_if);
+  else
+    k_cut_digits<false><<<blocksA + blocksB, 256, 0, st>>>(oA, oB, g.K, (int)Kp, blocksA, g.run_if);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   EmuShape s;
