@@ -114,6 +114,23 @@ ite_status ite_k_split(ite_ctx ctx, const double* X, int m, int n, int chi_max, 
                        int centre_right, double* left, double* right, double* sigma, int* rank,
                        double* discarded, int flags);
 
+/* ite_k_split with one of the guards of its preconditioner made to act, for tests (the
+ * paper has no counterpart; guard == 0 is ite_k_split).  The guards compare values in
+ * device memory, and this call changes the value; nothing faults or waits.  The result
+ * is a split to the same accuracy; blocks of fewer than 16 rows have no preconditioner
+ * and so no guards.
+ *   ITE_GUARD_WAIT        the block Jacobi's error word is set, as an expired wait sets it
+ *   ITE_GUARD_UNUSABLE    its rotation V is multiplied by 1.5: V is dropped
+ *   ITE_GUARD_THIRD_STEP  V is multiplied by 1.0001: a third Newton-Schulz step
+ *   ITE_GUARD_CORRECTION  every FP64 correction is refused */
+#define ITE_GUARD_WAIT 1
+#define ITE_GUARD_UNUSABLE 2
+#define ITE_GUARD_THIRD_STEP 3
+#define ITE_GUARD_CORRECTION 4
+ite_status ite_k_split_selftest(ite_ctx ctx, const double* X, int m, int n, int chi_max,
+                                double cutoff, int centre_right, double* left, double* right,
+                                double* sigma, int* rank, double* discarded, int flags, int guard);
+
 /* Self-test of the bounded grid-wide wait that the cooperative kernels of the
  * SVD (LQ and Jacobi sweeps) meet at after each step or round; the paper has
  * no counterpart.  Launches `blocks` co-resident blocks (2 <= blocks <= the

@@ -426,6 +426,18 @@ def k_split(ctx, X, m, n, chi_max, cutoff, centre_right, left, right, sigma=None
     return r.value, disc.value
 
 
+SPLIT_GUARDS = {"none": 0, "wait": 1, "unusable": 2, "third_step": 3, "correction": 4}
+
+
+def k_split_selftest(ctx, X, m, n, chi_max, cutoff, centre_right, left, right, sigma, tc, guard):
+    """k_split with one of the preconditioner's guards made to act."""
+    r, disc = C.c_int(), C.c_double()
+    check(lib.ite_k_split_selftest(ctx.h, _p(X), m, n, chi_max, cutoff, 1 if centre_right else 0,
+                                   _p(left), _p(right), _p(sigma), C.byref(r), C.byref(disc),
+                                   1 if tc else 0, SPLIT_GUARDS[guard]), ctx.h)
+    return r.value, disc.value
+
+
 def k_barrier_selftest(ctx, blocks, absent):
     """ite_k_barrier_selftest; returns the status (ITE_OK, or ITE_ETIMEOUT
     when `absent` blocks never reach the barrier)."""

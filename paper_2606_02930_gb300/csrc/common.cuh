@@ -216,27 +216,28 @@ cudaError_t svd_lq_r(const cplx* W, const cplx* beta, int p, int q, cplx* R, cud
 // and the steps between the GEMMs, which the engine issues.  K[0..3] are k x k
 // matrices; ok, gate_n, gate, gate_w, gate_w2 are device words for GemmArgs::run_if
 // (V usable; a third Newton-Schulz step needed; a correction E to apply; its
-// square, its fourth power needed); err
-// is nonzero after a bounded wait ran out; act lists the rows left to the FP64
-// Jacobi (as jacobi_rows takes them).
+// square, its fourth power needed); act lists the rows left to the FP64 Jacobi (as
+// jacobi_rows takes them).
 struct SvdPre {
   void* rows32;
   cplx* K[4];
-  int *act, *ok, *gate_n, *gate, *gate_w, *gate_w2, *err;
+  int *act, *ok, *gate_n, *gate, *gate_w, *gate_w2;
   int* rexp;                   // powers of two next to the row norms, for GemmArgs::kexp
   unsigned int* ctl;
 };
 size_t svd_pre_bytes(int k, int p);
 SvdPre svd_pre_carve(void* ws, int k, int p);
 // K[0] = V (k x k) from the fp32 block Jacobi on the rows of R, rexp from R; clears
-// the control words.  One cooperative launch of clusters.
+// the control words (expired: the error word starts as an expired wait leaves it).
+// One cooperative launch of clusters.
 cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const double* anorm2,
-                           cudaStream_t st);
+                           bool expired, cudaStream_t st);
 // M = V V^H (k x k) becomes -(M - I) / 2; step 0 decides *ok, step 1 *gate_n
 cudaError_t svd_pre_orth(const SvdPre& s, cplx* M, int k, int step, cudaStream_t st);
-// E (k x k) and rexp from G = S S^H, and the gates
+// E (k x k) and rexp from G = S S^H, and the gates: E is applied up to |E|_inf = nu_max
+constexpr double kPreNuMax = 2e-3;
 cudaError_t svd_pre_corr(const SvdPre& s, const cplx* G, int k, double tol, const double* anorm2,
-                         double skip_rel, cplx* E, cudaStream_t st);
+                         double skip_rel, double nu_max, cplx* E, cudaStream_t st);
 // E += W / 2 - W2 / 8 as the gates say
 cudaError_t svd_pre_comb(const SvdPre& s, cplx* E, const cplx* W, const cplx* W2, int k,
                          cudaStream_t st);

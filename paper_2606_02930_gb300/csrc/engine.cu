@@ -69,7 +69,7 @@ struct HostRead {
   int counter;
   int pad;
   int lq_err;
-  int pre_err;
+  int pad2;
   unsigned int pairs[2];
   double disc;
   double res;
@@ -474,7 +474,7 @@ ite_status add_left(ite_ctx ctx, const cplx* D, cplx* Y, int k, int len, cplx* t
 // lists (svd_pre.cu has the method); R is scratch afterwards.  Its matrices lie
 // in the Krylov basis' workspace, which no split needs.
 ite_status precondition(ite_ctx ctx, cplx* R, cplx* S, int k, int p, const double* anorm2,
-                        double skip_rel, double tol, const int** act, const int** err) {
+                        double skip_rel, double tol, int guard, const int** act) {
   CS(buf_ensure(ctx, ctx->ws_V, svd_pre_bytes(k, p)));
   const SvdPre s = svd_pre_carve(ctx->ws_V.p, k, p);
   cplx *A = s.K[0], *B = s.K[1], *W = s.K[2], *W2 = s.K[3];
@@ -482,7 +482,10 @@ ite_status precondition(ite_ctx ctx, cplx* R, cplx* S, int k, int p, const doubl
     return gemm(ctx, k, k, len, Y, len, 1, false, Y, 1, len, true, G, k, C(1), C(0), nullptr, C(0),
                 1, 0, 0, 0, run_if);
   };
-  CK(svd_pre_rotate(s, R, k, p, anorm2, ctx->stream));
+  CK(svd_pre_rotate(s, R, k, p, anorm2, guard == ITE_GUARD_WAIT, ctx->stream));
+  if (guard == ITE_GUARD_UNUSABLE || guard == ITE_GUARD_THIRD_STEP)
+    CK(vec_axpby(A, A, C(guard == ITE_GUARD_UNUSABLE ? 0.5 : 1e-4), C(1), (long long)k * k,
+                 ctx->stream));
   for (int it = 0; it < 3; ++it) {
     const int* on = it == 0 ? nullptr : it == 1 ? s.ok : s.gate_n;
     CS(gram(A, k, B, on));
@@ -494,7 +497,8 @@ ite_status precondition(ite_ctx ctx, cplx* R, cplx* S, int k, int p, const doubl
   CK(vec_copy_if(S, R, (long long)k * p, s.ok, false, ctx->stream));
   for (int it = 0; it < 2; ++it) {
     CS(gram(S, p, B));
-    CK(svd_pre_corr(s, B, k, tol, anorm2, skip_rel, A, ctx->stream));
+    CK(svd_pre_corr(s, B, k, tol, anorm2, skip_rel, guard == ITE_GUARD_CORRECTION ? 0.0 : kPreNuMax,
+                    A, ctx->stream));
     CS(gemm(ctx, k, k, k, A, k, 1, false, A, k, 1, false, W, k, C(1), C(0), nullptr, C(0), 1, 0, 0,
             0, s.gate_w));
     CS(gemm(ctx, k, k, k, W, k, 1, false, W, k, 1, false, W2, k, C(1), C(0), nullptr, C(0), 1, 0, 0,
@@ -505,7 +509,6 @@ ite_status precondition(ite_ctx ctx, cplx* R, cplx* S, int k, int p, const doubl
   CS(gram(S, p, B));
   CK(svd_pre_list(s, B, k, tol, anorm2, skip_rel, ctx->stream));
   *act = s.act;
-  *err = s.err;
   return ITE_OK;
 }
 
@@ -516,7 +519,7 @@ ite_status precondition(ite_ctx ctx, cplx* R, cplx* S, int k, int p, const doubl
 // projection U_r^H Xr (one GEMM, on the tensor cores in the tensor-core mode).
 ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double cutoff,
                  bool centre_right, cplx* left, cplx* right, int* r_out, double* disc_out,
-                 double* sigma_out = nullptr) {
+                 double* sigma_out = nullptr, int guard = 0) {
   Scope sc(ctx, P_SVD);
   const bool tr = !centre_right;
   const int p = tr ? n : m, q = tr ? m : n;
@@ -558,13 +561,12 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
   // its rounds outweigh the GEMMs of the preconditioner
   cplx* D = R;          // Sigma U^H in the end; the other of R and W is free
   const int* act = nullptr;
-  const int* pre_err = nullptr;
   {
     Scope jacobi_scope(ctx, P_JACOBI);
     const double tol = std::max(1e-15, p * kEps);
     if (k >= kPreMinRows) {
       D = W;
-      CS(precondition(ctx, R, D, k, p, anorm2, skip_weight(cutoff), tol, &act, &pre_err));
+      CS(precondition(ctx, R, D, k, p, anorm2, skip_weight(cutoff), tol, guard, &act));
     }
     if (ctx->group && k >= 3) {
       // the same Jacobi, launched together with other contexts' splits
@@ -592,11 +594,8 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
                      ctx->stream));
   CK(cudaMemcpyAsync(&ctx->hr->steps, reinterpret_cast<int*>(ctx->dcounter) + 10, sizeof(int),
                      cudaMemcpyDeviceToHost, ctx->stream));
-  ctx->hr->pre_err = 0;
-  if (pre_err)
-    CK(cudaMemcpyAsync(&ctx->hr->pre_err, pre_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CS(sync(ctx));
-  if (ctx->hr->counter != 0 || ctx->hr->lq_err != 0 || ctx->hr->pre_err != 0)
+  if (ctx->hr->counter != 0 || ctx->hr->lq_err != 0)
     return fail(ctx, ITE_ETIMEOUT, "SVD grid barrier wait ran out");
   if (ctx->hr->steps != 0) return fail(ctx, ITE_ETIMEOUT, "tensor-core GEMM wait ran out");
   ctx->jacobi_sweeps_total += ctx->hr->pad;
@@ -2598,7 +2597,15 @@ ite_status ite_k_barrier_selftest(ite_ctx ctx, int blocks, int absent) {
 ite_status ite_k_split(ite_ctx ctx, const double* X, int m, int n, int chi_max, double cutoff,
                        int centre_right, double* left, double* right, double* sigma, int* rank,
                        double* discarded, int flags) {
-  if (!ctx || !X || !left || !right || m < 1 || n < 1 || chi_max < 1 || !(cutoff >= 0.0))
+  return ite_k_split_selftest(ctx, X, m, n, chi_max, cutoff, centre_right, left, right, sigma, rank,
+                              discarded, flags, 0);
+}
+
+ite_status ite_k_split_selftest(ite_ctx ctx, const double* X, int m, int n, int chi_max,
+                                double cutoff, int centre_right, double* left, double* right,
+                                double* sigma, int* rank, double* discarded, int flags, int guard) {
+  if (!ctx || !X || !left || !right || m < 1 || n < 1 || chi_max < 1 || !(cutoff >= 0.0) ||
+      guard < 0 || guard > ITE_GUARD_CORRECTION)
     return ITE_EINVAL;
   struct ModeGuard {
     ite_ctx c;
@@ -2609,7 +2616,7 @@ ite_status ite_k_split(ite_ctx ctx, const double* X, int m, int n, int chi_max, 
   int r = 0;
   double disc = 0.0;
   CS(split(ctx, (const cplx*)X, m, n, chi_max, cutoff, centre_right != 0, (cplx*)left, (cplx*)right,
-           &r, &disc, sigma));
+           &r, &disc, sigma, guard));
   CS(sync(ctx));
   if (rank) *rank = r;
   if (discarded) *discarded = disc;

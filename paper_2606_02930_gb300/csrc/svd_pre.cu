@@ -31,9 +31,10 @@
 // cut): the entries of (V diag d)_i are then what the terms of row i weigh, and the
 // singular values keep the relative accuracy of FP64 products (1e-15 in that case).
 // S is updated by small corrections D S rather than replaced by Q S.
-// Guards: V is dropped (S = R, all rows go to the Jacobi) unless
-// |V V^H - I|_inf < 1e-2, from which three Newton-Schulz steps reach rounding;
-// a correction is dropped unless |E|_inf <= 2e-3.
+// Guards: V is dropped (S = R, all rows go to the Jacobi) unless no bounded wait ran
+// out in k_jacobi32 and |V V^H - I|_inf < 1e-2, from which three Newton-Schulz steps
+// reach rounding; a correction is dropped unless |E|_inf <= 2e-3.  What a guard drops
+// costs time, not the result: the FP64 Jacobi takes the rows that are left.
 #include <cooperative_groups.h>
 
 #include <mutex>
@@ -690,7 +691,6 @@ __global__ void k_copy_if(cplx* y, const cplx* x, long long n, const unsigned in
 }
 
 constexpr double kPairTan = 2.5e-4;           // tangents above this are left to the Jacobi
-constexpr double kNuMax = 2e-3;
 
 // E from G = S S^H: E_ij = -sign(D) t g_ij / |g_ij| (D = G_jj - G_ii, t the tangent of
 // the rotation that makes the pair orthogonal), exactly anti-Hermitian because
@@ -699,7 +699,7 @@ constexpr double kNuMax = 2e-3;
 // 4e-9, E^4 above 1e-4.
 __global__ void __launch_bounds__(RT)
 k_pre_corr(const cplx* __restrict__ G, int k, double tol, const double* anorm2, double skip_rel,
-           cplx* __restrict__ E, int* rexp, unsigned int* ctl) {
+           double nu_max, cplx* __restrict__ E, int* rexp, unsigned int* ctl) {
   const int i = blockIdx.x;
   const double skip = skip_rel * *anorm2;
   const double al = G[(long long)i * k + i].x;
@@ -729,7 +729,7 @@ k_pre_corr(const cplx* __restrict__ G, int k, double tol, const double* anorm2, 
   if (max_over_blocks(s, ctl, C_NU) && threadIdx.x == 0) {
     unsigned long long* w = reinterpret_cast<unsigned long long*>(ctl + C_NU);
     const double nu = __longlong_as_double((long long)__ldcg(w));
-    const bool on = nu > 0.0 && nu <= kNuMax;
+    const bool on = nu > 0.0 && nu <= nu_max;
     ctl[C_GE] = on;
     ctl[C_GW] = on && nu > 4e-9;
     ctl[C_GW2] = on && nu > 1e-4;
@@ -902,15 +902,18 @@ SvdPre svd_pre_carve(void* ws, int k, int p) {
   s.gate = reinterpret_cast<int*>(s.ctl + C_GE);
   s.gate_w = reinterpret_cast<int*>(s.ctl + C_GW);
   s.gate_w2 = reinterpret_cast<int*>(s.ctl + C_GW2);
-  s.err = reinterpret_cast<int*>(s.ctl + C_ERR);
   return s;
 }
 
 cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const double* anorm2,
-                           cudaStream_t st) {
+                           bool expired, cudaStream_t st) {
   const PreDims d = pre_dims(k, p);
   cudaError_t err = cudaMemsetAsync(s.ctl, 0, ctl_bytes(d), st);
   if (err != cudaSuccess) return err;
+  if (expired) {
+    err = cudaMemsetAsync(s.ctl + C_ERR, 1, sizeof(unsigned int), st);
+    if (err != cudaSuccess) return err;
+  }
   Pre32 a;
   a.R = static_cast<float2*>(s.rows32);
   a.V = a.R + (size_t)d.kp * d.pl;
@@ -965,9 +968,9 @@ cudaError_t vec_copy_if(cplx* y, const cplx* x, long long n, const int* flag, bo
 }
 
 cudaError_t svd_pre_corr(const SvdPre& s, const cplx* G, int k, double tol, const double* anorm2,
-                         double skip_rel, cplx* E, cudaStream_t st) {
+                         double skip_rel, double nu_max, cplx* E, cudaStream_t st) {
   count_launches(1);
-  k_pre_corr<<<k, RT, 0, st>>>(G, k, tol, anorm2, skip_rel, E, s.rexp, s.ctl);
+  k_pre_corr<<<k, RT, 0, st>>>(G, k, tol, anorm2, skip_rel, nu_max, E, s.rexp, s.ctl);
   return cudaGetLastError();
 }
 
