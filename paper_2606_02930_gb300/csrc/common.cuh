@@ -116,6 +116,8 @@ cudaError_t heff_lp_apply(const void* ops, const MixPlan& plan2, int d, int D0, 
 // zgemm_emu_scratch_bytes(M, N, K, entries of A, of B) bytes (an operand shared by
 // the batch has one); *err set if a bounded wait ran out.
 size_t zgemm_emu_scratch_bytes(int M, int N, int K, int batchA = 1, int batchB = 1);
+// false if the digit rows of the whole batch are more than one launch's tensor maps take
+bool zgemm_emu_rows_fit(int M, int N, int batchA, int batchB);
 cudaError_t zgemm_emu(const GemmArgs& g, void* scratch, size_t scratch_bytes, int* err,
                       cudaStream_t st);
 

@@ -210,6 +210,22 @@ ite_status buf_ensure(ite_ctx ctx, Buf& b, size_t bytes) {
   return ITE_OK;
 }
 
+// The same where less room is enough: *room says whether `bytes` could be had; if
+// not, the buffer is as large as it was.
+ite_status buf_try(ite_ctx ctx, Buf& b, size_t bytes, bool* room) {
+  *room = true;
+  if (b.n >= bytes && (b.p || bytes == 0)) return ITE_OK;
+  const size_t before = b.p ? b.n : 0;
+  buf_free(ctx, b);
+  b.p = dev_alloc(ctx, bytes);
+  if (b.p) {
+    b.n = bytes;
+    return ITE_OK;
+  }
+  *room = false;
+  return before ? buf_ensure(ctx, b, before) : ITE_OK;
+}
+
 template <typename T>
 T* P(Buf& b) { return reinterpret_cast<T*>(b.p); }
 
@@ -294,10 +310,27 @@ ite_status gemm(ite_ctx ctx, int M, int N, int K, const cplx* A, long long sAm, 
   g.C = Cm; g.ldc = ldc; g.sCb = sCb;
   g.alpha = alpha; g.beta = beta; g.Z = Z; g.gamma = gamma;
   if (emulated(ctx, M, N, K)) {
-    CS(buf_ensure(ctx, ctx->ws_emu,
-                  zgemm_emu_scratch_bytes(M, N, K, sAb ? batch : 1, sBb ? batch : 1)));
-    CK(zgemm_emu(g, ctx->ws_emu.p, ctx->ws_emu.n, reinterpret_cast<int*>(ctx->dcounter) + 10,
-                 ctx->stream));
+    int* err = reinterpret_cast<int*>(ctx->dcounter) + 10;
+    const int nbA = sAb ? batch : 1, nbB = sBb ? batch : 1;
+    const size_t all = zgemm_emu_scratch_bytes(M, N, K, nbA, nbB);
+    bool room = zgemm_emu_rows_fit(M, N, nbA, nbB);
+    if (room && batch > 1) CS(buf_try(ctx, ctx->ws_emu, all, &room));
+    else if (room) CS(buf_ensure(ctx, ctx->ws_emu, all));
+    if (room || batch == 1) {
+      CK(zgemm_emu(g, ctx->ws_emu.p, ctx->ws_emu.n, err, ctx->stream));
+      return ITE_OK;
+    }
+    // no room for the digits of the whole batch: one entry at a time
+    CS(buf_ensure(ctx, ctx->ws_emu, zgemm_emu_scratch_bytes(M, N, K)));
+    for (int b = 0; b < batch; ++b) {
+      GemmArgs e = g;
+      e.batch = 1;
+      e.A += b * sAb;
+      e.B += b * sBb;
+      e.C += b * sCb;
+      if (e.Z) e.Z += b * sCb;
+      CK(zgemm_emu(e, ctx->ws_emu.p, ctx->ws_emu.n, err, ctx->stream));
+    }
     return ITE_OK;
   }
   CK(zgemm(g, ctx->stream));

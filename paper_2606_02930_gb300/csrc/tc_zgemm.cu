@@ -587,6 +587,10 @@ size_t zgemm_emu_scratch_bytes(int M, int N, int K, int batchA, int batchB) {
          ((size_t)M * batchA + (size_t)N * batchB) * sizeof(int) + 1024;
 }
 
+bool zgemm_emu_rows_fit(int M, int N, int batchA, int batchB) {
+  return 2LL * S * M * batchA <= (1LL << 31) && (long long)S * N * batchB <= (1LL << 31);
+}
+
 cudaError_t zgemm_emu(const GemmArgs& g, void* scratch, size_t scratch_bytes, int* err,
                       cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
@@ -594,8 +598,7 @@ cudaError_t zgemm_emu(const GemmArgs& g, void* scratch, size_t scratch_bytes, in
   if (scratch_bytes < zgemm_emu_scratch_bytes(g.M, g.N, g.K, nbA, nbB)) return cudaErrorInvalidValue;
   const long long Kp = padded_k(g.K);
   const long long Mr = 2LL * g.M;
-  if ((long long)S * Mr * nbA > (1LL << 31) || (long long)S * g.N * nbB > (1LL << 31))
-    return cudaErrorInvalidValue;
+  if (!zgemm_emu_rows_fit(g.M, g.N, nbA, nbB)) return cudaErrorInvalidValue;
   __nv_bfloat16* As = reinterpret_cast<__nv_bfloat16*>(scratch);
   __nv_bfloat16* Bs = As + (size_t)S * Mr * nbA * Kp;
   int* eA = reinterpret_cast<int*>(Bs + (size_t)S * g.N * nbB * Kp);
