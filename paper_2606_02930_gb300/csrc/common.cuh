@@ -199,7 +199,8 @@ cudaError_t gmres_finish(GmresState* s, cudaStream_t st);
 // One cooperative launch; dev_state (8 device words) gets a nonzero word 4 if
 // a grid-barrier wait ran out.
 // refl (device, 3 k doubles, may be NULL) receives each reflector's
-// (Re u_0, Im u_0, c) for lq_formq.  pub (k q complex) is scratch.
+// (Re u_0, Im u_0, c) for lq_formq.  pub (k q complex) is scratch; without it (NULL)
+// the slower kernel that needs none runs.
 cudaError_t svd_lq(cplx* W, int p, int q, cplx* beta, double* refl, cplx* pub,
                    unsigned int* dev_state, cudaStream_t st);
 // L (p x k, row-major) with Xr = L Q^H from the output of svd_lq

@@ -505,10 +505,9 @@ ite_status add_left(ite_ctx ctx, const cplx* D, cplx* Y, int k, int len, cplx* t
 
 // S (k x p) = U R with U unitary and the rows of S orthogonal up to what act
 // lists (svd_pre.cu has the method); R is scratch afterwards.  Its matrices lie
-// in the Krylov basis' workspace, which no split needs.
+// in the Krylov basis' workspace (room for svd_pre_bytes), which no split needs.
 ite_status precondition(ite_ctx ctx, cplx* R, cplx* S, int k, int p, const double* anorm2,
                         double skip_rel, double tol, int guard, const int** act) {
-  CS(buf_ensure(ctx, ctx->ws_V, svd_pre_bytes(k, p)));
   const SvdPre s = svd_pre_carve(ctx->ws_V.p, k, p);
   cplx *A = s.K[0], *B = s.K[1], *W = s.K[2], *W2 = s.K[3];
   auto gram = [&](const cplx* Y, int len, cplx* G, const int* run_if = nullptr) {
@@ -575,6 +574,23 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
   unsigned int* jstate = reinterpret_cast<unsigned int*>(ctx->dcounter) + 16;
   unsigned int* lqstate = reinterpret_cast<unsigned int*>(ctx->dcounter) + 40;
   double* anorm2 = ctx->dscal + 8;
+  // Room that makes the split faster, in the Krylov basis' workspace and the digit
+  // buffer: the LQ's published rows and the preconditioner.  A split also runs
+  // without, so that it does not need more memory than its factors and their
+  // projection, whose digits come first.
+  bool lq_room = true, pre_room = k >= kPreMinRows;
+  {
+    const int r = std::min(k, chi_max);
+    auto digits = [&](int M, int N, int K) {
+      return emulated(ctx, M, N, K) ? zgemm_emu_scratch_bytes(M, N, K) : (size_t)0;
+    };
+    const size_t pub = (size_t)k * q * sizeof(cplx), proj = tr ? digits(m, r, n) : digits(r, n, m);
+    const size_t pre = std::max({proj, digits(k, p, k), digits(k, k, p), digits(k, k, k)});
+    if (pre_room) CS(buf_try(ctx, ctx->ws_emu, pre, &pre_room));
+    if (!pre_room) CS(buf_try(ctx, ctx->ws_emu, proj, &lq_room));
+    if (pre_room) CS(buf_try(ctx, ctx->ws_V, std::max(pub, svd_pre_bytes(k, p)), &pre_room));
+    if (!pre_room && lq_room) CS(buf_try(ctx, ctx->ws_V, pub, &lq_room));
+  }
   if (tr) CK(conj_transpose(X, m, n, W, ctx->stream));
   else CK(vec_copy(W, X, (long long)m * n, ctx->stream));
   CK(scaled_norm2(W, (long long)p * q, 1.0, anorm2, ctx->dscal + 16, ctx->stream));
@@ -586,8 +602,8 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
     for (int j = 0; j < k; ++j) f += 4.0 * (q - j) + 16.0 * (q - j) * (p - j - 1);
     ctx->lq_flops += f;
     Scope lq_scope(ctx, P_LQ, f);
-    CS(buf_ensure(ctx, ctx->ws_V, (size_t)k * q * sizeof(cplx)));
-    CK(svd_lq(W, p, q, beta, nullptr, P<cplx>(ctx->ws_V), lqstate, ctx->stream));
+    CK(svd_lq(W, p, q, beta, nullptr, lq_room ? P<cplx>(ctx->ws_V) : nullptr, lqstate,
+              ctx->stream));
   }
   CK(svd_lq_r(W, beta, p, q, R, ctx->stream));
   // 3. one-sided Jacobi on the k rows (length p) of R, preconditioned where
@@ -597,7 +613,7 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
   {
     Scope jacobi_scope(ctx, P_JACOBI);
     const double tol = std::max(1e-15, p * kEps);
-    if (k >= kPreMinRows) {
+    if (pre_room) {
       D = W;
       CS(precondition(ctx, R, D, k, p, anorm2, skip_weight(cutoff), tol, guard, &act));
     }
@@ -990,8 +1006,9 @@ ite_status gauge_lq(ite_ctx ctx, const cplx* X, int m, int n, cplx* left, cplx* 
   double* inv2 = ctx->dscal + 10;
   CK(vec_copy(W, X, (long long)m * n, ctx->stream));
   CK(scaled_norm2(W, (long long)m * n, 1.0, anorm2, ctx->dscal + 16, ctx->stream));
-  CS(buf_ensure(ctx, ctx->ws_V, (size_t)k * n * sizeof(cplx)));
-  CK(svd_lq(W, m, n, beta, refl, P<cplx>(ctx->ws_V), lqstate, ctx->stream));
+  bool room = false;
+  CS(buf_try(ctx, ctx->ws_V, (size_t)k * n * sizeof(cplx), &room));
+  CK(svd_lq(W, m, n, beta, refl, room ? P<cplx>(ctx->ws_V) : nullptr, lqstate, ctx->stream));
   CK(lq_inv_fnorm2(W, beta, n, k, colnorm, inv2, ctx->stream));
   CK(cudaMemcpyAsync(&ctx->hr->d[2], anorm2, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaMemcpyAsync(&ctx->hr->d[3], inv2, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));

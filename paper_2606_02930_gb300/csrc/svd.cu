@@ -1351,12 +1351,17 @@ cudaError_t svd_lq(cplx* W, int p, int q, cplx* beta, double* refl, cplx* pub,
   err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (err != cudaSuccess) return err;
   bool tried = false;
-  if (q <= 2 * LT) err = launch_lq_resident<2>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
-  else if (q <= 4 * LT) err = launch_lq_resident<4>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
-  else if (q <= 8 * LT) err = launch_lq_resident<8>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
-  else if (q <= 16 * LT) err = launch_lq_resident<16>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
+  if (pub && q <= 2 * LT)
+    err = launch_lq_resident<2>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
+  else if (pub && q <= 4 * LT)
+    err = launch_lq_resident<4>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
+  else if (pub && q <= 8 * LT)
+    err = launch_lq_resident<8>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
+  else if (pub && q <= 16 * LT)
+    err = launch_lq_resident<16>(W, p, q, beta, refl, pub, dev_state, sms, st, &tried);
   if (tried || err != cudaSuccess) return err;
-  // larger blocks: the rows in L2, one grid barrier per step
+  // larger blocks, or no room for the published rows: the rows in L2, one grid barrier
+  // per step
   int max_blocks = 0;
   err = g_lq_blocks.get((const void*)k_lq_persistent, JT, &max_blocks);
   if (err != cudaSuccess) return err;
