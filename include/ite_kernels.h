@@ -114,6 +114,11 @@ ite_status ite_k_split(ite_ctx ctx, const double* X, int m, int n, int chi_max, 
                        int centre_right, double* left, double* right, double* sigma, int* rank,
                        double* discarded, int flags);
 
+/* Occupancy queries that the splits have made of the driver since the library was
+ * loaded, over all contexts, for tests (the paper has no counterpart).  Each device is
+ * asked once per cluster size, whatever the sizes of the blocks. */
+long long ite_k_occupancy_queries(void);
+
 /* ite_k_split with one of the guards of its preconditioner made to act, for tests (the
  * paper has no counterpart; guard == 0 is ite_k_split).  The guards compare values in
  * device memory, and this call changes the value; nothing faults or waits.  The result

@@ -229,6 +229,7 @@ struct SvdPre {
   unsigned int* ctl;
 };
 size_t svd_pre_bytes(int k, int p);
+long long svd_pre_queries();   // occupancy queries made so far
 SvdPre svd_pre_carve(void* ws, int k, int p);
 // K[0] = V (k x k) from the fp32 block Jacobi on the rows of R, rexp from R; clears
 // the control words (expired: the error word starts as an expired wait leaves it).

@@ -2644,6 +2644,8 @@ ite_status ite_k_barrier_selftest(ite_ctx ctx, int blocks, int absent) {
   return ITE_OK;
 }
 
+long long ite_k_occupancy_queries(void) { return svd_pre_queries(); }
+
 ite_status ite_k_split(ite_ctx ctx, const double* X, int m, int n, int chi_max, double cutoff,
                        int centre_right, double* left, double* right, double* sigma, int* rank,
                        double* discarded, int flags) {

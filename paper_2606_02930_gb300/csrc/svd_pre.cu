@@ -37,7 +37,7 @@
 // costs time, not the result: the FP64 Jacobi takes the rows that are left.
 #include <cooperative_groups.h>
 
-#include <mutex>
+#include <atomic>
 
 #include "common.cuh"
 
@@ -827,15 +827,14 @@ constexpr size_t kFixedSmem = (size_t)PM * (4 * GLD + QLD) * sizeof(float2);
 constexpr int kChunkMax = 640;                // columns staged at once: 32 x 642 x 8 B = 164 KB
 constexpr size_t kOwnSmSmem = 116 * 1024;     // more than half of an SM's shared memory
 
-// Clusters of C CTAs with this much shared memory that can be resident at
-// once on the current device, cached per (device, C, bytes); several host
-// threads may ask at once.
-struct ClusterCapacity {
-  std::mutex mu;
-  struct Entry { int dev, C; size_t smem; int n; };
-  Entry e[64];
-  int used = 0;
-} g_cap;
+// Clusters of C CTAs that can be resident at once, per device and C (0: not asked yet;
+// two host threads may ask at once and get the same answer).  Asked at the largest
+// shared memory: every size in use is more than half of an SM's, so the answer is one
+// CTA per SM for all of them.
+constexpr size_t kMaxSmem = kFixedSmem + (size_t)PM * (kChunkMax + 2) * sizeof(float2);
+constexpr int kMaxCluster = 8, kMaxDevices = 64;
+std::atomic<int> g_capacity[kMaxDevices][kMaxCluster + 1];
+std::atomic<long long> g_queries{0};
 
 void launch_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int grid, int C, size_t smem,
                    cudaStream_t st, bool coop) {
@@ -853,29 +852,28 @@ void launch_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int grid, i
   cfg->numAttrs = coop ? 2 : 1;
 }
 
-cudaError_t cluster_capacity(int C, size_t smem, int* n) {
+cudaError_t cluster_capacity(int C, int* n) {
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
-  std::lock_guard<std::mutex> lock(g_cap.mu);
-  for (int i = 0; i < g_cap.used; ++i)
-    if (g_cap.e[i].dev == dev && g_cap.e[i].C == C && g_cap.e[i].smem == smem) {
-      *n = g_cap.e[i].n;
-      return cudaSuccess;
-    }
-  err = cudaFuncSetAttribute(k_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(kFixedSmem + (size_t)PM * (kChunkMax + 2) * sizeof(float2)));
+  std::atomic<int>& known = g_capacity[dev % kMaxDevices][C];
+  *n = known.load();
+  if (*n > 0) return cudaSuccess;
+  err = cudaFuncSetAttribute(k_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
   if (err != cudaSuccess) return err;
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute at[2];
-  launch_config(&cfg, at, C * 1024, C, smem, nullptr, false);
+  launch_config(&cfg, at, C * 1024, C, kMaxSmem, nullptr, false);
+  g_queries.fetch_add(1);
   err = cudaOccupancyMaxActiveClusters(n, k_jacobi32, &cfg);
   if (err != cudaSuccess) return err;
-  if (g_cap.used < 64) g_cap.e[g_cap.used++] = {dev, C, smem, *n};
+  known.store(*n);
   return cudaSuccess;
 }
 
 }  // namespace
+
+long long svd_pre_queries() { return g_queries.load(); }
 
 size_t svd_pre_bytes(int k, int p) {
   const PreDims d = pre_dims(k, p);
@@ -928,7 +926,7 @@ cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const d
   // as many CTAs per pair as give every CTA an SM of its own (two on one SM
   // take turns at every phase of the step)
   const int pairs = a.nb / 2;
-  int C = 8, cap = 0;
+  int C = kMaxCluster, cap = 0;
   size_t smem = 0;
   for (;; --C) {
     a.pc = share(p, C);
@@ -936,7 +934,7 @@ cudaError_t svd_pre_rotate(const SvdPre& s, const cplx* R, int k, int p, const d
     a.chunk = a.pc + a.vc < kChunkMax ? a.pc + a.vc : kChunkMax;
     smem = kFixedSmem + (size_t)PM * (a.chunk + 2) * sizeof(float2);
     if (smem < kOwnSmSmem) smem = kOwnSmSmem;
-    err = cluster_capacity(C, smem, &cap);
+    err = cluster_capacity(C, &cap);
     if (err != cudaSuccess) return err;
     if (cap >= pairs || C == 1) break;
   }

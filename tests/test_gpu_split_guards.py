@@ -62,3 +62,16 @@ def test_guard_out_of_range_is_refused(api, ctx):
         st = _lib.lib.ite_k_split_selftest(ctx.h, X.data_ptr(), 20, 20, 20, 0.0, 1, X.data_ptr(),
                                            X.data_ptr(), None, None, None, 0, guard)
         assert st == _lib.ITE_EINVAL
+
+
+def test_occupancy_is_asked_once_per_cluster_size(api, ctx):
+    # 70 lengths of the rows, each with a shared memory of its own
+    import torch
+    from paper_2606_02930_gb300 import _lib
+    out = torch.empty(5000 * 16, dtype=torch.complex128, device="cuda")
+    right = torch.empty(256, dtype=torch.complex128, device="cuda")
+    X = to_dev(crandn(np.random.default_rng(1), 5000, 16))
+    before = _lib.lib.ite_k_occupancy_queries()
+    for m in range(2400, 2400 + 70 * 32, 32):
+        api.k_split(ctx, X, m, 16, 16, 0.0, True, out, right)
+    assert _lib.lib.ite_k_occupancy_queries() - before <= 8
