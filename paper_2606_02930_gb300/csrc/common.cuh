@@ -56,6 +56,8 @@ struct GemmArgs {
   const int* kexp = nullptr;
 };
 cudaError_t zgemm(const GemmArgs& g, cudaStream_t st);
+// SMs of the current device (asked once per device)
+cudaError_t device_sms(int* sms);
 
 // ---------------------------------------------------------------- tensor cores
 // C[M][N] (fp32, leading dimension ldc) = A[M][K] B[N][K]^T with A, B bf16

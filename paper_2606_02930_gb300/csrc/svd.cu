@@ -1345,10 +1345,8 @@ cudaError_t svd_lq(cplx* W, int p, int q, cplx* beta, double* refl, cplx* pub,
   cudaError_t err = cudaMemsetAsync(dev_state, 0, 8 * sizeof(unsigned int), st);
   if (err != cudaSuccess) return err;
   if (p < 1 || q < 1) return cudaSuccess;
-  int sms = 0, dev = 0;
-  err = cudaGetDevice(&dev);
-  if (err != cudaSuccess) return err;
-  err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int sms = 0;
+  err = device_sms(&sms);
   if (err != cudaSuccess) return err;
   bool tried = false;
   if (pub && q <= 2 * LT)

@@ -603,16 +603,9 @@ cudaError_t zgemm_emu(const GemmArgs& g, void* scratch, size_t scratch_bytes, in
   __nv_bfloat16* Bs = As + (size_t)S * Mr * nbA * Kp;
   int* eA = reinterpret_cast<int*>(Bs + (size_t)S * g.N * nbB * Kp);
   int* eB = eA + (size_t)g.M * nbA;
-  static std::atomic<int> sm_count[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  int sms = 0;
+  cudaError_t e = device_sms(&sms);
   if (e != cudaSuccess) return e;
-  int sms = sm_count[dev & 63].load();
-  if (sms == 0) {
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    sm_count[dev & 63].store(sms);
-  }
   const Operand oA = {g.A, g.sAm, g.sAk, g.sAb, g.conjA ? 1 : 0, g.M, nbA, As, eA,
                       g.kexp, 1};
   const Operand oB = {g.B, g.sBn, g.sBk, g.sBb, g.conjB ? 1 : 0, g.N, nbB, Bs, eB,

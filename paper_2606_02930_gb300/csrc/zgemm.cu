@@ -14,6 +14,8 @@
 // SMs idle: 347 us, against 33 us of FP64 work spread over the GPU.  One small
 // H_eff (chi = 32) 250 -> 55 us, GMRES(10) at chi = 64 5.55 -> 1.91 ms (with the
 // MPO mix's change).
+#include <atomic>
+
 #include "common.cuh"
 
 namespace ite {
@@ -183,20 +185,35 @@ void launch_conj(const GemmArgs& g, bool a_kfast, bool b_nfast, cudaStream_t st)
 
 // Work of the busiest SM in outputs, if the tiles are dealt evenly, with what a
 // small tile costs more per output (fewer products per load).
-double busiest(const GemmArgs& g, int T, double factor) {
+double busiest(const GemmArgs& g, int T, double factor, int sms) {
   const double tiles = (double)((g.M + T - 1) / T) * ((g.N + T - 1) / T) * g.batch;
-  const double sms = 152.0;
   return factor * T * T * (double)(long long)((tiles + sms - 1.0) / sms);
 }
 
 }  // namespace
+
+cudaError_t device_sms(int* sms) {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  *sms = known[dev & 63].load();
+  if (*sms > 0) return cudaSuccess;
+  err = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+  if (err == cudaSuccess) known[dev & 63].store(*sms);
+  return err;
+}
 
 cudaError_t zgemm(const GemmArgs& g, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return cudaSuccess;
   if (g.batch > 65535 || (g.M + BM - 1) / BM > 65535) return cudaErrorInvalidValue;
   const bool a_kfast = (g.sAk == 1);
   const bool b_nfast = (g.sBn == 1) || (g.sBk != 1);
-  const double w32 = busiest(g, 32, 1.0), w16 = busiest(g, 16, 1.1), w8 = busiest(g, 8, 1.25);
+  int sms = 0;
+  const cudaError_t err = device_sms(&sms);
+  if (err != cudaSuccess) return err;
+  const double w32 = busiest(g, 32, 1.0, sms), w16 = busiest(g, 16, 1.1, sms),
+               w8 = busiest(g, 8, 1.25, sms);
   count_launches(1);
   if ((w32 <= w16 && w32 <= w8) || (g.M + 7) / 8 > 65535) launch_conj<32>(g, a_kfast, b_nfast, st);
   else if (w16 <= w8) launch_conj<16>(g, a_kfast, b_nfast, st);
