@@ -190,6 +190,21 @@ double busiest(const GemmArgs& g, int T, double factor, int sms) {
   return factor * T * T * (double)(long long)((tiles + sms - 1.0) / sms);
 }
 
+// C shares memory with A or B (as intervals of addresses).
+bool in_place(const GemmArgs& g) {
+  struct Span { const cplx *lo, *hi; };
+  auto span = [&](const cplx* p, long long n0, long long s0, long long n1, long long s1,
+                  long long sb) {
+    Span r = {p, p + 1};
+    const long long d[3] = {(n0 - 1) * s0, (n1 - 1) * s1, (g.batch - 1) * sb};
+    for (long long x : d) (x < 0 ? r.lo : r.hi) += x;
+    return r;
+  };
+  const Span a = span(g.A, g.M, g.sAm, g.K, g.sAk, g.sAb), b = span(g.B, g.K, g.sBk, g.N, g.sBn, g.sBb);
+  const Span c = span(g.C, g.M, g.ldc, g.N, 1, g.sCb);
+  return (c.lo < a.hi && a.lo < c.hi) || (c.lo < b.hi && b.lo < c.hi);
+}
+
 }  // namespace
 
 cudaError_t device_sms(int* sms) {
@@ -214,8 +229,11 @@ cudaError_t zgemm(const GemmArgs& g, cudaStream_t st) {
   if (err != cudaSuccess) return err;
   const double w32 = busiest(g, 32, 1.0, sms), w16 = busiest(g, 16, 1.1, sms),
                w8 = busiest(g, 8, 1.25, sms);
+  // a product of one 32 x 32 tile reads its operands in full before it writes, so it
+  // may write over one of them; smaller tiles would read what others have written
+  const bool one_tile = g.M <= BM && g.N <= BN && in_place(g);
   count_launches(1);
-  if ((w32 <= w16 && w32 <= w8) || (g.M + 7) / 8 > 65535) launch_conj<32>(g, a_kfast, b_nfast, st);
+  if ((w32 <= w16 && w32 <= w8) || (g.M + 7) / 8 > 65535 || one_tile) launch_conj<32>(g, a_kfast, b_nfast, st);
   else if (w16 <= w8) launch_conj<16>(g, a_kfast, b_nfast, st);
   else launch_conj<8>(g, a_kfast, b_nfast, st);
   return cudaGetLastError();

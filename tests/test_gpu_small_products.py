@@ -62,3 +62,24 @@ def test_heff_with_dense_mpo(api, ctx, D, d, cplx):
     Y = to_dev(np.zeros((chlB, d, d, chrB), complex))
     api.k_heff(ctx, H, 1, to_dev(L_to_lib(L)), to_dev(R_to_lib(R)), to_dev(X), Y)
     assert rel_err(to_host(Y), want) < 1e-12
+
+
+@pytest.mark.parametrize("n,m", [(20, 20), (32, 32), (9, 30)])
+@pytest.mark.parametrize("left", [True, False])
+def test_small_product_in_place(api, ctx, n, m, left):
+    # C on top of an operand, while other work takes the SMs in turns with the product's
+    # blocks: a block that wrote before another had read would show
+    import torch
+    rng = np.random.default_rng(n + m)
+    busy = torch.randn(1 << 28, dtype=torch.float64, device="cuda")
+    side = torch.cuda.Stream()
+    X = crandn(rng, n, m)
+    F = crandn(rng, n, n) if left else crandn(rng, m, m)
+    want = F @ X if left else X @ F
+    Fd = to_dev(F)
+    for _ in range(150):
+        C = to_dev(X)
+        with torch.cuda.stream(side):
+            torch.sin(torch.sin(busy))
+        api.k_zgemm(ctx, *((Fd, C) if left else (C, Fd)), C, mode=0)
+        assert np.abs(to_host(C) - want).max() <= 8 * 36 * 2.0 ** -52 * np.abs(F).max() * np.abs(X).max()
