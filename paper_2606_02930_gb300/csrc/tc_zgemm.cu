@@ -169,14 +169,14 @@ k_zgemm_slices(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   uint64_t* acc_full = empty + STAGES;
   uint64_t* acc_empty = acc_full + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
-  __shared__ int s_fail;
+  __shared__ int s_fail, s_loads, s_mmas;       // K tiles whose loads, MMAs were issued
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nkb = g.nkb;
   const int nchunk = (nkb + KB_PER_CHUNK - 1) / KB_PER_CHUNK;
 
   if (threadIdx.x == 0) {
-    s_fail = 0;
+    s_fail = s_loads = s_mmas = 0;
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
@@ -227,6 +227,7 @@ k_zgemm_slices(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           tma_load_4d(st + S * A_SLICE, &tmB, &full[s], kb * BK, n0, g.b_batched ? b : 0);
         }
       }
+      s_loads = it;
     }
   } else if (warp == T::EW + 1) {
     // ---- MMA issuer
@@ -274,6 +275,7 @@ k_zgemm_slices(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
         }
       }
+      s_mmas = it;
     }
   } else {
     // ---- epilogue warps: TMEM lane quarter warp % 4, columns 32 (warp / 4)..
@@ -342,10 +344,18 @@ k_zgemm_slices(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
       }
     }
-    if (!ok && lane == 0) atomicExch(g.err, 1);
+    if (!ok && lane == 0) s_fail = 1;
   }
   __syncthreads();
-  if (s_fail && threadIdx.x == 0) atomicExch(g.err, 1);
+  // after a wait that ran out: the last loads and MMAs of each stage (bounded), so that
+  // none is in flight when the block's memory is given back
+  if (s_fail && threadIdx.x == 0) {
+    atomicExch(g.err, 1);
+    for (int it = max(s_loads - STAGES, 0); it < s_loads; ++it)
+      mbar_wait(&full[it % STAGES], (it / STAGES) & 1);
+    for (int it = max(s_mmas - STAGES, 0); it < s_mmas; ++it)
+      mbar_wait(&empty[it % STAGES], (it / STAGES) & 1);
+  }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
