@@ -114,6 +114,13 @@ ite_status ite_k_split(ite_ctx ctx, const double* X, int m, int n, int chi_max, 
                        int centre_right, double* left, double* right, double* sigma, int* rank,
                        double* discarded, int flags);
 
+/* The fp32 rotation of the splits' block Jacobi for n pairs of rows, for its test (the
+ * paper has no counterpart): rows of squared norms alpha[i], beta[i] (at most 1) and
+ * inner product g[2i] + i g[2i+1] = x y^dag give c[i] and s[2i] + i s[2i+1] with
+ * x' = c x - s y and y' = conj(s) x + c y orthogonal.  All pointers are to the device. */
+ite_status ite_k_rotation_selftest(ite_ctx ctx, int n, const float* alpha, const float* beta,
+                                   const float* g, float* c, float* s);
+
 /* Occupancy queries that the splits have made of the driver since the library was
  * loaded, over all contexts, for tests (the paper has no counterpart).  Each device is
  * asked once per cluster size, whatever the sizes of the blocks. */

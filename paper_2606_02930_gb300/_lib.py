@@ -139,6 +139,7 @@ SIGNATURES = {
     "ite_k_zgemm": (_i, [_vp, _i, _i, _i, _i, _vp, C.c_longlong, C.c_longlong, _i, _vp,
                          C.c_longlong, C.c_longlong, _i, _vp, C.c_longlong, _pd, _pd]),
     "ite_k_split": (_i, [_vp, _vp, _i, _i, _i, _d, _i, _vp, _vp, _vp, _pi, _pd, _i]),
+    "ite_k_rotation_selftest": (_i, [_vp, _i, _vp, _vp, _vp, _vp, _vp]),
     "ite_k_occupancy_queries": (C.c_longlong, []),
     "ite_k_split_selftest": (_i, [_vp, _vp, _i, _i, _i, _d, _i, _vp, _vp, _vp, _pi, _pd, _i, _i]),
     "ite_k_barrier_selftest": (_i, [_vp, _i, _i]),

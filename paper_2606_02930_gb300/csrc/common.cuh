@@ -231,6 +231,8 @@ struct SvdPre {
   unsigned int* ctl;
 };
 size_t svd_pre_bytes(int k, int p);
+cudaError_t svd_pre_rotations(int n, const float* al, const float* be, const float* g, float* c,
+                              float* s, cudaStream_t st);
 long long svd_pre_queries();   // occupancy queries made so far
 SvdPre svd_pre_carve(void* ws, int k, int p);
 // K[0] = V (k x k) from the fp32 block Jacobi on the rows of R, rexp from R; clears

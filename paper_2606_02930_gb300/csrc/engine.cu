@@ -2644,6 +2644,13 @@ ite_status ite_k_barrier_selftest(ite_ctx ctx, int blocks, int absent) {
   return ITE_OK;
 }
 
+ite_status ite_k_rotation_selftest(ite_ctx ctx, int n, const float* alpha, const float* beta,
+                                   const float* g, float* c, float* s) {
+  if (!ctx || n < 1 || !alpha || !beta || !g || !c || !s) return ITE_EINVAL;
+  CK(svd_pre_rotations(n, alpha, beta, g, c, s, ctx->stream));
+  return sync(ctx);
+}
+
 long long ite_k_occupancy_queries(void) { return svd_pre_queries(); }
 
 ite_status ite_k_split(ite_ctx ctx, const double* X, int m, int n, int chi_max, double cutoff,
