@@ -170,8 +170,12 @@ ite_status ite_profile_start(ite_ctx ctx);
  * the same algorithmic count as category 0, which they are not part of). */
 ite_status ite_profile_stop(ite_ctx ctx, double ms[ITE_PROFILE_SLOTS],
                             double flops[ITE_PROFILE_SLOTS], long long counts[ITE_PROFILE_SLOTS]);
+/* Splits that were preconditioned and the sweeps of their fp32 block Jacobi, since the
+ * last call (then reset); either pointer may be NULL. */
+ite_status ite_svd_sweeps32(ite_ctx ctx, long long* splits, long long* sweeps);
 /* SVD statistics since the last call (then reset): splits performed, total
- * and largest number of Jacobi sweeps, and (fp64_flops, may be NULL; three
+ * and largest number of sweeps of the FP64 Jacobi (on the rows that the
+ * preconditioner leaves to it), and (fp64_flops, may be NULL; three
  * entries) the algorithmic FP64 flops of the Householder LQ ([0]), of the
  * Jacobi rotations and inner products actually executed ([1]), and the
  * reference algorithmic work of the truncated SVDs ([2]: 8.7 GFLOP for a

@@ -468,6 +468,13 @@ def profile_stop(ctx):
             for i, k in enumerate(PROFILE_CATEGORIES)}
 
 
+def svd_sweeps32(ctx):
+    """(preconditioned splits, mean sweeps of their fp32 block Jacobi) since the last call."""
+    splits, sweeps = C.c_longlong(), C.c_longlong()
+    check(lib.ite_svd_sweeps32(ctx.h, C.byref(splits), C.byref(sweeps)), ctx.h)
+    return splits.value, sweeps.value / max(1, splits.value)
+
+
 def svd_stats(ctx):
     splits, total, mx = C.c_longlong(), C.c_longlong(), C.c_int()
     fl = np.zeros(3)

@@ -228,6 +228,7 @@ struct SvdPre {
   cplx* K[4];
   int *act, *ok, *gate_n, *gate, *gate_w, *gate_w2;
   int* rexp;                   // powers of two next to the row norms, for GemmArgs::kexp
+  const int* sweeps;           // sweeps of the fp32 block Jacobi
   unsigned int* ctl;
 };
 size_t svd_pre_bytes(int k, int p);

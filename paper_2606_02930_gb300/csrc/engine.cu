@@ -69,7 +69,7 @@ struct HostRead {
   int counter;
   int pad;
   int lq_err;
-  int pad2;
+  int sweeps32;
   unsigned int pairs[2];
   double disc;
   double res;
@@ -114,6 +114,7 @@ struct ite_ctx_s {
   long long jacobi_sweeps_total = 0, jacobi_splits = 0;
   double jacobi_flops = 0.0, lq_flops = 0.0, svd_alg_flops = 0.0;
   int jacobi_sweeps_max = 0;
+  long long pre_sweeps = 0, pre_splits = 0;    // of the fp32 block Jacobi
   // event profiling of the sweep's stages (off unless started)
   bool prof = false;
   std::vector<cudaEvent_t> evpool;
@@ -507,7 +508,7 @@ ite_status add_left(ite_ctx ctx, const cplx* D, cplx* Y, int k, int len, cplx* t
 // lists (svd_pre.cu has the method); R is scratch afterwards.  Its matrices lie
 // in the Krylov basis' workspace (room for svd_pre_bytes), which no split needs.
 ite_status precondition(ite_ctx ctx, cplx* R, cplx* S, int k, int p, const double* anorm2,
-                        double skip_rel, double tol, int guard, const int** act) {
+                        double skip_rel, double tol, int guard, const int** act, const int** sweeps32) {
   const SvdPre s = svd_pre_carve(ctx->ws_V.p, k, p);
   cplx *A = s.K[0], *B = s.K[1], *W = s.K[2], *W2 = s.K[3];
   auto gram = [&](const cplx* Y, int len, cplx* G, const int* run_if = nullptr) {
@@ -541,6 +542,7 @@ ite_status precondition(ite_ctx ctx, cplx* R, cplx* S, int k, int p, const doubl
   CS(gram(S, p, B));
   CK(svd_pre_list(s, B, k, tol, anorm2, skip_rel, ctx->stream));
   *act = s.act;
+  *sweeps32 = s.sweeps;
   return ITE_OK;
 }
 
@@ -610,12 +612,13 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
   // its rounds outweigh the GEMMs of the preconditioner
   cplx* D = R;          // Sigma U^H in the end; the other of R and W is free
   const int* act = nullptr;
+  const int* sweeps32 = nullptr;
   {
     Scope jacobi_scope(ctx, P_JACOBI);
     const double tol = std::max(1e-15, p * kEps);
     if (pre_room) {
       D = W;
-      CS(precondition(ctx, R, D, k, p, anorm2, skip_weight(cutoff), tol, guard, &act));
+      CS(precondition(ctx, R, D, k, p, anorm2, skip_weight(cutoff), tol, guard, &act, &sweeps32));
     }
     if (ctx->group && k >= 3) {
       // the same Jacobi, launched together with other contexts' splits
@@ -643,12 +646,18 @@ ite_status split(ite_ctx ctx, const cplx* X, int m, int n, int chi_max, double c
                      ctx->stream));
   CK(cudaMemcpyAsync(&ctx->hr->steps, reinterpret_cast<int*>(ctx->dcounter) + 10, sizeof(int),
                      cudaMemcpyDeviceToHost, ctx->stream));
+  if (sweeps32)
+    CK(cudaMemcpyAsync(&ctx->hr->sweeps32, sweeps32, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CS(sync(ctx));
   if (ctx->hr->counter != 0 || ctx->hr->lq_err != 0)
     return fail(ctx, ITE_ETIMEOUT, "SVD grid barrier wait ran out");
   if (ctx->hr->steps != 0) return fail(ctx, ITE_ETIMEOUT, "tensor-core GEMM wait ran out");
   ctx->jacobi_sweeps_total += ctx->hr->pad;
   ctx->jacobi_splits += 1;
+  if (sweeps32) {
+    ctx->pre_sweeps += ctx->hr->sweeps32;
+    ctx->pre_splits += 1;
+  }
   ctx->jacobi_sweeps_max = std::max(ctx->jacobi_sweeps_max, ctx->hr->pad);
   // FP64 flops of the Jacobi as the device ran it: 8 per element and examined
   // pair (one inner product; the row norms are tracked), 20 per element and
@@ -1469,6 +1478,14 @@ ite_status ite_svd_stats(ite_ctx ctx, long long* splits, long long* sweeps_total
   return ITE_OK;
 }
 
+ite_status ite_svd_sweeps32(ite_ctx ctx, long long* splits, long long* sweeps) {
+  if (!ctx) return ITE_EINVAL;
+  if (splits) *splits = ctx->pre_splits;
+  if (sweeps) *sweeps = ctx->pre_sweeps;
+  ctx->pre_splits = ctx->pre_sweeps = 0;
+  return ITE_OK;
+}
+
 ite_status ite_profile_start(ite_ctx ctx) {
   if (!ctx) return ITE_EINVAL;
   ctx->prof = true;
@@ -1755,6 +1772,9 @@ ite_status step_impl(ite_ctx ctx, ite_mpo H, ite_mps psi, double dtau, int schem
         ctx->jacobi_flops += cc->jacobi_flops;
         ctx->lq_flops += cc->lq_flops;
         ctx->svd_alg_flops += cc->svd_alg_flops;
+        ctx->pre_sweeps += cc->pre_sweeps;
+        ctx->pre_splits += cc->pre_splits;
+        cc->pre_sweeps = cc->pre_splits = 0;
         cc->jacobi_sweeps_total = cc->jacobi_splits = 0;
         cc->jacobi_sweeps_max = 0;
         cc->jacobi_flops = cc->lq_flops = cc->svd_alg_flops = 0.0;

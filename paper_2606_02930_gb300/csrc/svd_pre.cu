@@ -916,6 +916,7 @@ SvdPre svd_pre_carve(void* ws, int k, int p) {
   s.rexp = s.act + 2 * k + 1;
   s.ctl = reinterpret_cast<unsigned int*>(take(ctl_bytes(d)));
   s.ok = reinterpret_cast<int*>(s.ctl + C_OK);
+  s.sweeps = reinterpret_cast<const int*>(s.ctl + C_SWEEPS);
   s.gate_n = reinterpret_cast<int*>(s.ctl + C_GN);
   s.gate = reinterpret_cast<int*>(s.ctl + C_GE);
   s.gate_w = reinterpret_cast<int*>(s.ctl + C_GW);

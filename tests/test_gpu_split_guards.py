@@ -75,3 +75,15 @@ def test_occupancy_is_asked_once_per_cluster_size(api, ctx):
     for m in range(2400, 2400 + 70 * 32, 32):
         api.k_split(ctx, X, m, 16, 16, 0.0, True, out, right)
     assert _lib.lib.ite_k_occupancy_queries() - before <= 8
+
+
+def test_fp32_sweeps_are_counted(api, ctx):
+    import torch
+    X = to_dev(crandn(np.random.default_rng(2), 64, 64))
+    left, right = torch.empty_like(X), torch.empty_like(X)
+    api.svd_sweeps32(ctx)
+    for n in (64, 64, 12):          # the last has too few rows to be preconditioned
+        api.k_split(ctx, X, n, n, n, 0.0, True, left, right)
+    splits, mean = api.svd_sweeps32(ctx)
+    assert splits == 2 and 1 <= mean <= 16
+    assert api.svd_sweeps32(ctx) == (0, 0.0)
