@@ -104,12 +104,16 @@ ite_status ite_k_local_solve(ite_ctx ctx, ite_mpo H, int i, int chl, int chr, co
  * singular values for the first chi_max entries down to a squared weight of
  * 1e-3 max(cutoff, 1e-25) of the total.  Rows that cannot be kept (below that
  * weight, or far below the chi_max-th) are not resolved among themselves, so
- * beyond those entries only the sum of squares is exact.  Algorithm: Householder LQ of the rows on the isometry side; from 16
- * rows an fp32 block Jacobi whose rotation, made unitary in FP64, and two
- * FP64 corrections orthogonalise the rows of the triangular factor; one-sided
- * FP64 Jacobi on the rows left; projection GEMM.  flags bit 0 runs the
- * projection GEMM on the tensor cores with FP64-class accuracy (the emulation
- * of ite_k_zgemm mode 1). */
+ * beyond those entries only the sum of squares is exact.  Algorithm:
+ * Householder LQ of the rows on the isometry side; from 16 rows an fp32 block
+ * Jacobi whose rotation, made unitary in FP64, and two FP64 corrections
+ * orthogonalise the rows of the triangular factor; one-sided FP64 Jacobi on the
+ * rows left; projection GEMM.  flags bit 0 runs the projection GEMM and the
+ * products of the rotation and the corrections, where they are large enough, on
+ * the tensor cores with FP64-class accuracy (the emulation of ite_k_zgemm mode 1).
+ * The factors and sigma then differ from those without it by rounding; light
+ * singular values of graded blocks keep their relative accuracy either way.
+ * Without device memory for the preconditioner all rows go to the FP64 Jacobi. */
 ite_status ite_k_split(ite_ctx ctx, const double* X, int m, int n, int chi_max, double cutoff,
                        int centre_right, double* left, double* right, double* sigma, int* rank,
                        double* discarded, int flags);

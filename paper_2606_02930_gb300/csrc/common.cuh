@@ -34,6 +34,27 @@ __host__ __device__ __forceinline__ void cfma_conj(cplx& acc, cplx a, cplx b) {
 
 namespace ite {
 
+#ifdef __CUDACC__
+// v[0..8) summed over the warp: the lanes with lane % 4 == 0 return sum lane / 4
+// (half of what a lane holds goes at each exchange: 9 adds instead of 40)
+__device__ __forceinline__ double warp_sum8(double (&v)[8]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int n = 4, m = 16; n >= 1; n >>= 1, m >>= 1) {
+    const bool up = (lane & m) != 0;
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const double send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+    }
+  }
+  double r = v[0];
+  r += __shfl_xor_sync(0xffffffffu, r, 2);
+  r += __shfl_xor_sync(0xffffffffu, r, 1);
+  return r;
+}
+#endif
+
 // Number of kernels this library has launched (process-wide, all contexts).
 void count_launches(unsigned long long n);
 unsigned long long launches();

@@ -4,8 +4,8 @@
 // side whose isometry is wanted, the split runs
 //   1. a Householder LQ of the rows, Xr H_0 H_1 ... H_{k-1} = L (p x k lower
 //      trapezoidal, k = min(p, q)), all k reflector steps in one cooperative
-//      launch: k_lq_resident holds the rows in registers or shared memory,
-//      k_lq_persistent is for rows that fit in neither;
+//      launch: k_lq_resident holds the rows in shared memory, k_lq_persistent is
+//      for rows that do not fit there;
 //   2. R = L^H (k x p, upper trapezoidal), so that R^H R = Xr Xr^H: the rows
 //      of R carry the left singular structure of Xr and are graded like its
 //      singular values, which is what lets the Jacobi below converge in few
@@ -190,25 +190,6 @@ __device__ __forceinline__ bool load_pub(const cplx* p, cplx& v) {
   asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
   v = cmake(__longlong_as_double((long long)a), __longlong_as_double((long long)b));
   return a != kUnset && b != kUnset;
-}
-
-// v[0..8) summed over the warp: the lanes with lane % 4 == 0 return sum lane / 4
-// (half of what a lane holds goes at each exchange: 9 adds instead of 40)
-__device__ __forceinline__ double warp_sum8(double (&v)[8]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int n = 4, m = 16; n >= 1; n >>= 1, m >>= 1) {
-    const bool up = (lane & m) != 0;
-#pragma unroll
-    for (int i = 0; i < n; ++i) {
-      const double send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
-    }
-  }
-  double r = v[0];
-  r += __shfl_xor_sync(0xffffffffu, r, 2);
-  r += __shfl_xor_sync(0xffffffffu, r, 1);
-  return r;
 }
 
 // One element of a row per thread and LT columns: EPT >= q / LT

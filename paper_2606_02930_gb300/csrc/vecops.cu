@@ -252,25 +252,6 @@ int arnoldi_grid(long long n) {
   return (int)(g > 608 ? 608 : g < 1 ? 1 : g);
 }
 
-// Sums v[0..8) over the warp; the lanes with lane % 4 == 0 return sum number
-// (lane >> 2) (bits 4, 3, 2 of the lane select the half kept at each exchange).
-__device__ __forceinline__ double warp_sum8(double (&v)[8]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int n = 4, m = 16; n >= 1; n >>= 1, m >>= 1) {
-    const bool up = (lane & m) != 0;
-#pragma unroll
-    for (int i = 0; i < n; ++i) {
-      const double send = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
-    }
-  }
-  double r = v[0];
-  r += __shfl_xor_sync(0xffffffffu, r, 2);
-  r += __shfl_xor_sync(0xffffffffu, r, 1);
-  return r;
-}
-
 // sh[warp][2 i], sh[warp][2 i + 1] = this warp's share of conj(V_i) . w over the
 // elements of its threads
 __device__ __forceinline__ void dot_shares(const cplx* V, long long ldv, int nv, const cplx* w,
