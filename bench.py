@@ -37,7 +37,7 @@ TAU0, TAU_MAX, K_GRID = 1e-3, 1e3, 40
 SEED = 2000
 METRIC = "H_eff matvec TFLOP/s; τ-steps/s vs plain FP64 at equal ΔE; p50/p99 latency"
 UNIT = "tau-steps/s"
-# FP64 pipe of GB300 (no measured FP64 peak exists for this machine): 152 SMs x
+# FP64 pipe of GB300 (derived, there is no measured FP64 peak): 152 SMs x
 # 2 DFMA/clk x 2 FLOP x 2.07 GHz = 1.26 TFLOP/s, in line with the nominal
 # 1.25 TFLOP/s (a DFMA probe measured 1.19 at 1995 MHz).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
