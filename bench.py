@@ -631,7 +631,8 @@ def run_ours(args, rank, world, local_rank):
             "stage_ms_per_step": breakdown,
             "step_ms": [round(x, 3) for x in step_ms],
             "heff_calls_per_step": heff["count"] // max(1, args.steps),
-            "svd_jacobi": svd,
+            "svd_jacobi": {"what": "FP64 Jacobi on the rows that the preconditioner leaves",
+                           **svd},
             "energies": [i["energy"] for i in infos],
             "clocks": clk}
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
