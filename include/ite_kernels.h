@@ -125,7 +125,7 @@ ite_status ite_k_split(ite_ctx ctx, const double* X, int m, int n, int chi_max, 
 ite_status ite_k_rotation_selftest(ite_ctx ctx, int n, const float* alpha, const float* beta,
                                    const float* g, float* c, float* s);
 
-/* Occupancy queries that the splits have made of the driver since the library was
+/* Occupancy queries that the splits have made of CUDA since the library was
  * loaded, over all contexts, for tests (the paper has no counterpart).  Each device is
  * asked once per cluster size, whatever the sizes of the blocks. */
 long long ite_k_occupancy_queries(void);
